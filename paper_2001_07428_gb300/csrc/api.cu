@@ -95,11 +95,12 @@ struct Phase {
   OpDev op{};
   OpDev opdf{};           // double-float phase, stencil: (hi, lo) links for the Lanczos products
   bool dfmv = false;      // use opdf for the Lanczos products
-  void* V = nullptr;      // n x (m + 1); float4 (hi, lo) pairs in a double-float phase
-  void* Vtmp = nullptr;   // n x kk (rotation target; FP64 in a double-float phase)
+  void* V = nullptr;      // n x (m + 1): FP32, (hi, lo) float4 pairs (df), or the fixed-point basis (fx)
+  void* Vtmp = nullptr;   // n x kk (rotation target; FP64 but in the FP32 phase)
   void* y = nullptr;      // the vector being built
-  void* x = nullptr;      // double-float phase: FP64 copy of v_j (the matvec input)
+  void* x = nullptr;      // df, fx: v_j in FP64 (the matvec input)
   bool df = false;        // basis stored as compensated FP32 pairs
+  bool fx = false;        // basis stored in fixed point (plain FP64; fixed.cuh)
   size_t cs = 0;          // bytes per complex number of V
   double* alpha_part = nullptr;
   double* resid_part = nullptr;
@@ -133,6 +134,9 @@ struct jtrlan_ctx {
   double* part_dot = nullptr;
   double* part_nrm = nullptr;
   coef4* coef = nullptr;
+  int* vexp = nullptr;             // exponents of the basis columns (GSArgs)
+  int* kmax = nullptr;             // scratch of launch_store_cols
+  int* part_max = nullptr;
   StepState* st = nullptr;
   double* d_res = nullptr;
   double* d_candlam = nullptr;
@@ -151,7 +155,7 @@ struct jtrlan_ctx {
   int* h_order = nullptr;
   double* h_misc = nullptr;
   int gs_nblk = 0, gs_rpb = 0;
-  int coop64 = 0, coop32 = 0, coopdf = 0;   // row blocks (= CTAs) of the cooperative Gram-Schmidt step; 0: not used
+  int coopfx = 0, coop32 = 0, coopdf = 0;   // row blocks (= CTAs) of the cooperative Gram-Schmidt step; 0: not used
   int coop_rpb = 0, coop_rpb_df = 0;        // its rows per block
   bool invert = false;             // Algorithm 1's invert mode: the Lanczos product is A^{-1} v by CG
   void *cg_r = nullptr, *cg_p = nullptr, *cg_q = nullptr;   // CG residual, direction, A p
@@ -344,7 +348,9 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
     return JTRLAN_OK;
   };
   if (!c->mixed) {
+    c->p64.fx = true;
     JT_TRY(make_phase(c->p64, sizeof(double2)));
+    JT_TRY(c->dalloc(&c->p64.x, (size_t)c->n * sizeof(double2)));
   } else {  // double-float phase on the FP64 operator
     c->pdf.op = o;
     c->pdf.df = true;
@@ -454,7 +460,8 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
     int per = 0;
     if (!c->mixed) {
       JT_CUDA(gs_coop_occupancy<double>(m, &per));
-      if (per > 0) part(per, &c->coop_rpb, &c->coop64, 1);
+      // up to 32 tiles of rows go to eight blocks, one thread-block cluster (gsfx.cu)
+      if (per > 0) part(per, &c->coop_rpb, &c->coopfx, tiles <= 32 ? (tiles + 7) / 8 : 1);
     }
     if (prm->precision == JTRLAN_MIXED) {
       JT_CUDA(gs_coop_occupancy<float>(m, &per));
@@ -482,8 +489,8 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
       }
     }
   }
-  if (prm->gs_split) c->coop64 = c->coop32 = c->coopdf = 0;   // the separate-launch Gram-Schmidt path
-  const int nblk_max = std::max(c->gs_nblk, std::max(std::max(c->coop64, c->coop32), c->coopdf));
+  if (prm->gs_split) c->coopfx = c->coop32 = c->coopdf = 0;   // the separate-launch Gram-Schmidt path
+  const int nblk_max = std::max(c->gs_nblk, std::max(std::max(c->coopfx, c->coop32), c->coopdf));
   JT_TRY(c->dalloc(&c->T, (size_t)(m + 1) * (m + 1) * sizeof(double)));
   JT_TRY(c->dalloc(&c->lam, (size_t)m * sizeof(double)));
   JT_TRY(c->dalloc(&c->Z, (size_t)m * m * sizeof(double)));
@@ -492,6 +499,9 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
   JT_TRY(c->dalloc(&c->part_dot, (size_t)(m + 1) * nblk_max * sizeof(coef4)));
   JT_TRY(c->dalloc(&c->part_nrm, (size_t)2 * nblk_max * sizeof(double)));   // two slots (cooperative step)
   JT_TRY(c->dalloc(&c->coef, (size_t)(m + 1) * sizeof(coef4)));
+  JT_TRY(c->dalloc(&c->vexp, (size_t)(m + 1) * sizeof(int)));
+  JT_TRY(c->dalloc(&c->kmax, (size_t)(m + 1) * sizeof(int)));
+  JT_TRY(c->dalloc(&c->part_max, (size_t)2 * nblk_max * sizeof(int)));
   JT_TRY(c->dalloc(&c->st, sizeof(StepState)));
   JT_TRY(c->dalloc(&c->d_res, (size_t)c->nev * sizeof(double)));
   JT_TRY(c->dalloc(&c->d_candlam, (size_t)c->nev * sizeof(double)));
@@ -607,9 +617,9 @@ jtrlan_status filter_apply_cert_io(jtrlan_ctx* c, Phase& ph, const void* v64, co
   return JTRLAN_OK;
 }
 
+// y = p(A) v_j; v_j in FP64 is ph.x.
 jtrlan_status filter_apply_cert(jtrlan_ctx* c, Phase& ph, int j) {
-  const void* vj = col(ph.V, c->n, j, ph.cs);
-  return filter_apply_cert_io(c, ph, ph.df ? ph.x : vj, vj, ph.y);   // v_j in FP64: ph.x beside a (hi, lo) basis
+  return filter_apply_cert_io(c, ph, ph.x, col(ph.V, c->n, j, ph.cs), ph.y);
 }
 
 // Rayleigh quotient lam_out = x^H A x and residual res_out = ||A x - lam x|| of one FP64 column
@@ -716,7 +726,9 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
   cudaStream_t s = c->stream;
   const int64_t n = c->n;
   const size_t cs = ph.cs;
-  if (ph.df) LAUNCH(K_OTHER, launch_fp64_from_df(col(ph.V, n, j0, cs), ph.x, n, s));   // v_j0 in FP64
+  // v_j0 in FP64 for the first product
+  if (ph.df) LAUNCH(K_OTHER, launch_fp64_from_df(col(ph.V, n, j0, cs), ph.x, n, s));
+  if (ph.fx) LAUNCH(K_OTHER, launch_load_col(ph.V, c->vexp, n, j0, (double2*)ph.x, s));
   const int mv_parts = c->invert ? cg_blocks(n)
                        : (filtered && !(ph.certify && ph.dfmv)) ? cheb_blocks(n)
                        : ph.dfmv ? matvec_df_blocks(ph.opdf) : ph.mv_nblk;
@@ -729,10 +741,10 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
     } else if (ph.dfmv) {   // compensated FP32 on the (hi, lo) column and links, FP64 result
       LAUNCH(K_MATVEC, launch_matvec_df(ph.opdf, col(ph.V, n, j, cs), ph.y, ph.alpha_part, s));
     } else if (c->invert) {   // invert mode: y = A^{-1} v_j by CG, then the partials of v_j^H y
-      JT_TRY(cg_solve(c, ph, col(ph.V, n, j, cs), ph.y));
-      LAUNCH(K_CG, launch_vhy_part(col(ph.V, n, j, cs), ph.y, n, ph.alpha_part, s));
+      JT_TRY(cg_solve(c, ph, ph.x, ph.y));
+      LAUNCH(K_CG, launch_vhy_part(ph.x, ph.y, n, ph.alpha_part, s));
     } else {
-      const void* vj = ph.df ? ph.x : col(ph.V, n, j, cs);
+      const void* vj = ph.x ? ph.x : col(ph.V, n, j, cs);
       LAUNCH(K_MATVEC, launch_matvec<R>(ph.op, (const C*)vj, (C*)ph.y, MV_ALPHA, ph.alpha_part,
                                         nullptr, nullptr, 0, 0, nullptr, s));
     }
@@ -757,7 +769,7 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
       }
       LAUNCH(K_GS_NORMALIZE, launch_gsdf_normalize(a, ph.x, s));
     } else {
-      const int coop = std::is_same<R, float>::value ? c->coop32 : c->coop64;
+      const int coop = std::is_same<R, float>::value ? c->coop32 : c->coopfx;
       if (coop > 0) {   // the whole step in one cooperative launch, on its own row partition
         GSArgs ac = a;
         ac.nblk = coop;
@@ -768,11 +780,11 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
       }
       LAUNCH(K_GS_FIRST, launch_gs_first<R>(a, (const double2*)ph.alpha_part, mv_parts, s));
       LAUNCH(K_GS_REDUCE, launch_gs_reduce(a, 1, s));
-      LAUNCH(K_GS_UPDATE, launch_gs_update<R>(a, s));
+      LAUNCH(K_GS_UPDATE, launch_gs_update<R>(a, 1, s));
       for (int pass = 2; pass <= c->gs_passes; ++pass) {
         LAUNCH(K_GS_DOT, launch_gs_dot<R>(a, pass, s));
         LAUNCH(K_GS_REDUCE, launch_gs_reduce(a, 0, s));
-        LAUNCH(K_GS_UPDATE, launch_gs_update<R>(a, s));
+        LAUNCH(K_GS_UPDATE, launch_gs_update<R>(a, pass, s));
       }
       LAUNCH(K_GS_NORMALIZE, launch_gs_normalize<R>(a, s));
     }
@@ -798,6 +810,7 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
   a.V = ph.V; a.n = n; a.h = c->h; a.y = ph.y; a.part_dot = c->part_dot; a.part_nrm = c->part_nrm;
   a.coef = c->coef; a.st = c->st; a.T = c->T; a.ldt = ldt; a.m = m; a.nblk = c->gs_nblk;
   a.rows_per_block = c->gs_rpb;
+  a.vexp = c->vexp; a.part_max = c->part_max; a.x = (double2*)ph.x;
   a.no_w = c->prm.plain_trlan ? 1 : 0;
   const double mv_units = ph.op.kind == JTRLAN_STENCIL4D ? (double)ph.op.vol : (double)c->h * (double)c->h;
   ev.assign(nev, 0.0);
@@ -816,7 +829,7 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
     stt.n_matvec += (int64_t)(m - k) * per_step;                         // invert mode: A^{-1} v_j
     if (!c->invert) c->work[K_MATVEC] += (double)(m - k) * per_step * mv_units;
     if (c->invert) {   // c = ||A v_{m+1}|| of the invert-mode residual estimates (Algorithm 1)
-      const void* vm1 = col(ph.V, n, m, cs);
+      const void* vm1 = ph.x;   // v_{m+1}
       LAUNCH(K_CG, launch_matvec<double>(ph.op, (const double2*)vm1, (double2*)c->cg_q, MV_PLAIN, nullptr, nullptr,
                                          nullptr, 0, 0, nullptr, s));
       LAUNCH(K_CG, launch_resid_part(c->cg_q, vm1, &c->cg_st->zero, n, ph.resid_part, s));
@@ -840,8 +853,10 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
         LAUNCH(K_ROTATE, launch_rotate_tc(ph.V, n, m, Zc, ncols, out, c->tc, c0 == 0, s));
       else if (ph.df)
         LAUNCH(K_ROTATE, launch_rotate_df(ph.V, n, m, Zc, ncols, out, s));
+      else if (ph.fx)
+        LAUNCH(K_ROTATE, launch_rotate_fx(ph.V, c->vexp, n, m, Zc, ncols, out, s));
       else
-        LAUNCH(K_ROTATE, launch_rotate<R>(ph.V, n, m, Zc, ncols, out, s));
+        LAUNCH(K_ROTATE, launch_rotate<float>(ph.V, n, m, Zc, ncols, out, s));
       c->work[K_ROTATE] += 2.0 * (double)n * m * ncols;
       return JTRLAN_OK;
     };
@@ -891,9 +906,13 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
       // product (reading R6b).
       int hit = -1;
       if (res_est[i] < 1e-3 * tol_ph)
-        for (size_t q = 0; q < locked_ev.size(); ++q)
-          if (std::fabs(ev[i] - locked_ev[q]) <= 1e-12 * std::max(1.0, std::fabs(ev[i]))) { hit = (int)q; break; }
+        for (size_t q = 0; q < locked_ev.size(); ++q) {   // the nearest
+          const double d = std::fabs(ev[i] - locked_ev[q]);
+          if (d <= 1e-12 * std::max(1.0, std::fabs(ev[i])) && (hit < 0 || d < std::fabs(ev[i] - locked_ev[hit]))) hit = (int)q;
+        }
       if (hit >= 0) {
+        ev[i] = locked_ev[hit];           // to the last bit: the Ritz value comes back within an ulp or two
+        if (!c->invert) lamv[i] = ev[i];
         res[i] = locked_res[hit];
         rq[i] = locked_rq[hit];
         conv[i] = 1;
@@ -956,8 +975,8 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
       JT_CUDA(cudaMemcpyAsync(c->d_perm, c->h_perm, m * sizeof(int), cudaMemcpyHostToDevice, s));
       if (ph.df)
         LAUNCH(K_SHRINK, launch_shrink_df(ph.V, ph.Vtmp, n, c->d_perm, nev, m, s));
-      else
-        LAUNCH(K_SHRINK, launch_shrink<R>(ph.V, ph.Vtmp, n, c->d_perm, nev, m, s));
+      else if (!ph.fx)   // the pairs of a fixed-point basis are read from Vtmp
+        LAUNCH(K_SHRINK, launch_shrink<float>(ph.V, ph.Vtmp, n, c->d_perm, nev, m, s));
       JT_CUDA(cudaStreamSynchronize(s));
       JT_CUDA(c->prof.harvest());
       break;
@@ -980,8 +999,11 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
     JT_CUDA(cudaMemcpyAsync(c->d_perm, c->h_perm, m * sizeof(int), cudaMemcpyHostToDevice, s));
     if (ph.df)
       LAUNCH(K_SHRINK, launch_shrink_df(ph.V, ph.Vtmp, n, c->d_perm, k, m, s));  // and v_{k+1} = v_{m+1}
+    else if (ph.fx)
+      LAUNCH(K_SHRINK, launch_store_cols(ph.V, ph.Vtmp, n, c->d_perm, k, m, c->vexp, c->kmax, s));
     else
-      LAUNCH(K_SHRINK, launch_shrink<R>(ph.V, ph.Vtmp, n, c->d_perm, k, m, s));
+      LAUNCH(K_SHRINK, launch_shrink<float>(ph.V, ph.Vtmp, n, c->d_perm, k, m, s));
+    if (ph.fx) c->nl[K_SHRINK] += 1;   // two kernels
   }
   // carry the device counters of this phase into the next one
   c->work_base[0] = c->work[K_GS_FIRST];
@@ -1006,21 +1028,20 @@ jtrlan_status bounds_impl(jtrlan_ctx* c, int steps, double* lo, double* hi) {
   JT_CUDA(cudaMemsetAsync(c->st, 0, sizeof(StepState), s));
   JT_CUDA(cudaMemsetAsync(c->T, 0, (size_t)ldt * ldt * sizeof(double), s));
   const uint64_t seed = 0xb07d5ull;
-  if (ph.df) {
-    LAUNCH(K_OTHER, launch_fill_random<double>(ph.x, n, seed, s));
-    LAUNCH(K_OTHER, launch_normalize_col<double>(ph.x, n, c->part_nrm, c->gs_nblk, s));
-    LAUNCH(K_OTHER, launch_df_from_fp64(ph.x, ph.V, n, s));
-  } else if (fp32) {
+  if (fp32) {
     LAUNCH(K_OTHER, launch_fill_random<float>(ph.V, n, seed, s));
     LAUNCH(K_OTHER, launch_normalize_col<float>(ph.V, n, c->part_nrm, c->gs_nblk, s));
   } else {
-    LAUNCH(K_OTHER, launch_fill_random<double>(ph.V, n, seed, s));
-    LAUNCH(K_OTHER, launch_normalize_col<double>(ph.V, n, c->part_nrm, c->gs_nblk, s));
+    LAUNCH(K_OTHER, launch_fill_random<double>(ph.x, n, seed, s));
+    LAUNCH(K_OTHER, launch_normalize_col<double>(ph.x, n, c->part_nrm, c->gs_nblk, s));
+    if (ph.df) LAUNCH(K_OTHER, launch_df_from_fp64(ph.x, ph.V, n, s));
+    else LAUNCH(K_OTHER, launch_store_cols(ph.V, ph.x, n, nullptr, 1, 0, c->vexp, c->kmax, s));
   }
   GSArgs a{};
   a.V = ph.V; a.n = n; a.h = c->h; a.y = ph.y; a.part_dot = c->part_dot; a.part_nrm = c->part_nrm;
   a.coef = c->coef; a.st = c->st; a.T = c->T; a.ldt = ldt; a.m = c->m; a.nblk = c->gs_nblk;
   a.rows_per_block = c->gs_rpb;
+  a.vexp = c->vexp; a.part_max = c->part_max; a.x = (double2*)ph.x;
   a.no_w = c->prm.plain_trlan ? 1 : 0;
   if (fp32) JT_TRY(lanczos_steps<float>(c, ph, a, 0, steps, false));
   else JT_TRY(lanczos_steps<double>(c, ph, a, 0, steps, false));
@@ -1054,6 +1075,7 @@ jtrlan_status solve_impl(jtrlan_ctx* c, jtrlan_stats* stats_out) {
   std::vector<double> ev, res;
   int icnv = 0;
   jtrlan_status st = JTRLAN_OK;
+  Phase& final = c->mixed ? c->pdf : c->p64;
   if (c->prm.precision == JTRLAN_MIXED) {
     // FP32 phase: matvec, Gram-Schmidt and rotation in FP32, alpha/beta and Ritz in FP64, to the
     // tolerance max(tol, 1e-5 max|t|) that FP32 vectors can certify.
@@ -1077,27 +1099,23 @@ jtrlan_status solve_impl(jtrlan_ctx* c, jtrlan_stats* stats_out) {
     stt.n_restarts += s32.n_restarts;
     // the double-float phase starts from the normalised sum of the FP32 Ritz vectors (promoted)
     LAUNCH(K_OTHER, launch_sum_columns(ph.V, n, std::max(icnv, 1), c->pdf.x, s));
-  } else if (c->mixed) {
-    if (c->prm.v1)
-      JT_CUDA(cudaMemcpyAsync(c->pdf.x, c->prm.v1, (size_t)n * sizeof(double2), cudaMemcpyDefault, s));
-    else
-      LAUNCH(K_OTHER, launch_fill_ones<double>(c->pdf.x, n, s));
+  } else if (c->prm.v1) {
+    JT_CUDA(cudaMemcpyAsync(final.x, c->prm.v1, (size_t)n * sizeof(double2), cudaMemcpyDefault, s));
   } else {
-    if (c->prm.v1) {
-      JT_CUDA(cudaMemcpyAsync(c->p64.V, c->prm.v1, (size_t)n * sizeof(double2), cudaMemcpyDefault, s));
-      LAUNCH(K_OTHER, launch_normalize_col<double>(c->p64.V, n, c->part_nrm, c->gs_nblk, s));
-      c->nl[K_OTHER] += 1;  // two kernels
-    } else {
-      LAUNCH(K_OTHER, launch_fill_ones<double>(c->p64.V, n, s));  // v_1 = 1 / ||1||
-    }
+    LAUNCH(K_OTHER, launch_fill_ones<double>(final.x, n, s));   // v_1 = 1 / ||1||
   }
-  if (c->mixed) {  // normalise the FP64 start and store it split into the (hi, lo) basis
-    LAUNCH(K_OTHER, launch_normalize_col<double>(c->pdf.x, n, c->part_nrm, c->gs_nblk, s));
+  if (c->mixed || c->prm.v1) {
+    LAUNCH(K_OTHER, launch_normalize_col<double>(final.x, n, c->part_nrm, c->gs_nblk, s));
+    c->nl[K_OTHER] += 1;  // two kernels
+  }
+  if (final.df) {   // normalised; stored as the basis's first column
+    LAUNCH(K_OTHER, launch_df_from_fp64(final.x, final.V, n, s));
+  } else {
+    LAUNCH(K_OTHER, launch_store_cols(final.V, final.x, n, nullptr, 1, 0, c->vexp, c->kmax, s));
     c->nl[K_OTHER] += 1;
-    LAUNCH(K_OTHER, launch_df_from_fp64(c->pdf.x, c->pdf.V, n, s));
   }
   jtrlan_stats s64{};
-  st = run_phase<double>(c, c->mixed ? c->pdf : c->p64, c->prm.tol, 0.0, c->max_restarts, s64, ev, res, &icnv);
+  st = run_phase<double>(c, final, c->prm.tol, 0.0, c->max_restarts, s64, ev, res, &icnv);
   stt.n_matvec += s64.n_matvec;
   stt.n_resid_matvec += s64.n_resid_matvec;
   stt.n_gs_passes += s64.n_gs_passes;
@@ -1179,14 +1197,14 @@ jtrlan_status jtrlan_pairs(jtrlan_ctx* c, int with_partners, double* evals, void
       if (c->mixed)
         JT_CUDA(launch_gather_pairs_df(c->pdf.V, c->n, c->d_order, nev, with_partners, evecs, c->stream));
       else
-        JT_CUDA(launch_gather_pairs<double>(c->p64.V, c->n, c->d_order, nev, with_partners, evecs, c->stream));
+        JT_CUDA(launch_gather_pairs(c->p64.Vtmp, c->d_perm, c->n, c->d_order, nev, with_partners, evecs, c->stream));
     } else {
       void* tmp = nullptr;
       JT_CUDA(cudaMallocAsync(&tmp, bytes, c->stream));
       if (c->mixed)
         JT_CUDA(launch_gather_pairs_df(c->pdf.V, c->n, c->d_order, nev, with_partners, tmp, c->stream));
       else
-        JT_CUDA(launch_gather_pairs<double>(c->p64.V, c->n, c->d_order, nev, with_partners, tmp, c->stream));
+        JT_CUDA(launch_gather_pairs(c->p64.Vtmp, c->d_perm, c->n, c->d_order, nev, with_partners, tmp, c->stream));
       JT_CUDA(cudaMemcpyAsync(evecs, tmp, bytes, cudaMemcpyDeviceToHost, c->stream));
       JT_CUDA(cudaFreeAsync(tmp, c->stream));
     }

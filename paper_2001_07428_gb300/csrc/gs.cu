@@ -16,6 +16,7 @@
 // The data-dependent repeat runs without host synchronisation: every pass is launched, and each
 // kernel of a pass returns at once when the device-side flag st->done says the loop has exited.
 // All reductions use a fixed order, so results are reproducible run to run.
+// These kernels serve the FP32 basis; the FP64 ones are in gs64.cu.
 #include <cooperative_groups.h>
 
 #include "internal.h"
@@ -357,7 +358,7 @@ __global__ void scale_by_norm_kernel(cplx<R>* v, int64_t n, const double* part, 
   s = block_sum(s, sh);
   const R inv = (R)(1.0 / sqrt(s));
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    v[i] = cscale(v[i], inv);
+    v[i] = cadd(cscale(v[i], inv), mk<R>(0, 0));   // -0.0 becomes 0
 }
 
 template <typename R>
@@ -590,7 +591,7 @@ cudaError_t launch_gs_reduce(const GSArgs& a, int first, cudaStream_t s) {
 }
 
 template <typename R>
-cudaError_t launch_gs_update(const GSArgs& a, cudaStream_t s) {
+cudaError_t launch_gs_update(const GSArgs& a, int /*pass*/, cudaStream_t s) {
   gs_update_kernel<R><<<a.nblk, kGsThreads, (size_t)(a.j + 1) * sizeof(coef4), s>>>(a);
   return cudaGetLastError();
 }
@@ -681,20 +682,14 @@ cudaError_t launch_gs_step_coop(const GSArgs& a, const double2* alpha_part, int 
   return cudaLaunchCooperativeKernel((const void*)gs_step_coop_kernel<R>, dim3(grid), dim3(kGsThreads), args,
                                      gs_coop_smem<R>(a.m), s);
 }
-template cudaError_t gs_coop_occupancy<double>(int, int*);
 template cudaError_t gs_coop_occupancy<float>(int, int*);
-template cudaError_t launch_gs_step_coop<double>(const GSArgs&, const double2*, int, int, double*, int, cudaStream_t);
 template cudaError_t launch_gs_step_coop<float>(const GSArgs&, const double2*, int, int, double*, int, cudaStream_t);
-template cudaError_t launch_gs_first<double>(const GSArgs&, const double2*, int, cudaStream_t);
 template cudaError_t launch_gs_first<float>(const GSArgs&, const double2*, int, cudaStream_t);
-template cudaError_t launch_gs_update<float>(const GSArgs&, cudaStream_t);
+template cudaError_t launch_gs_update<float>(const GSArgs&, int, cudaStream_t);
 template cudaError_t launch_gs_dot<float>(const GSArgs&, int, cudaStream_t);
 template cudaError_t launch_gs_normalize<float>(const GSArgs&, cudaStream_t);
 template cudaError_t launch_fill_ones<float>(void*, int64_t, cudaStream_t);
 template cudaError_t launch_normalize_col<float>(void*, int64_t, double*, int, cudaStream_t);
-template cudaError_t launch_gs_update<double>(const GSArgs&, cudaStream_t);
-template cudaError_t launch_gs_dot<double>(const GSArgs&, int, cudaStream_t);
-template cudaError_t launch_gs_normalize<double>(const GSArgs&, cudaStream_t);
 template cudaError_t launch_fill_ones<double>(void*, int64_t, cudaStream_t);
 template cudaError_t launch_fill_random<double>(void*, int64_t, uint64_t, cudaStream_t);
 template cudaError_t launch_fill_random<float>(void*, int64_t, uint64_t, cudaStream_t);

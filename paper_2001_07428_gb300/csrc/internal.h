@@ -60,6 +60,10 @@ struct GSArgs {
   int nblk;            // blocks of the row-parallel GS kernels
   int no_w;            // nonzero: plain TRLAN (Gram-Schmidt against V only, W removed)
   int rows_per_block;  // row pairs per block (multiple of 32)
+  // the FP64 form (gsfx.cu), whose V is the fixed-point basis of fixed.cuh
+  int* vexp;           // [m+1] K of the columns: |v| < 2^(K - 1023)
+  int* part_max;       // [2][nblk] high words of the largest |component| of y
+  double2* x;          // v_j in FP64 (the product's input), rewritten with v_{j+1} by the normalisation
 };
 int gs_blocks(int64_t h, int* rows_per_block);
 
@@ -69,11 +73,28 @@ template <typename R>
 cudaError_t launch_gs_first(const GSArgs& a, const double2* alpha_part, int n_alpha_part, cudaStream_t s);
 cudaError_t launch_gs_reduce(const GSArgs& a, int first, cudaStream_t s);
 template <typename R>
-cudaError_t launch_gs_update(const GSArgs& a, cudaStream_t s);
+cudaError_t launch_gs_update(const GSArgs& a, int pass, cudaStream_t s);   // pass: 1 after the first dots
 template <typename R>
 cudaError_t launch_gs_dot(const GSArgs& a, int pass, cudaStream_t s);
 template <typename R>
 cudaError_t launch_gs_normalize(const GSArgs& a, cudaStream_t s);
+// the FP64 form on the fixed-point basis (gsfx.cu)
+template <> cudaError_t launch_gs_first<double>(const GSArgs&, const double2*, int, cudaStream_t);
+template <> cudaError_t launch_gs_update<double>(const GSArgs&, int, cudaStream_t);
+template <> cudaError_t launch_gs_dot<double>(const GSArgs&, int, cudaStream_t);
+template <> cudaError_t launch_gs_normalize<double>(const GSArgs&, cudaStream_t);
+// Columns of the fixed-point basis V (n x (m + 1)): store FP64 columns X[:, perm[c]] (perm null: c) as
+// V[:, 0..k) and, if k < m, V[:, m] as V[:, k]; load V[:, c] into x.  kmax: scratch
+// of k ints.
+cudaError_t launch_store_cols(void* V, const void* X, int64_t n, const int* perm, int k, int m, int* vexp, int* kmax,
+                              cudaStream_t s);
+cudaError_t launch_load_col(const void* V, const int* vexp, int64_t n, int c, double2* x, cudaStream_t s);
+// out[:, c] = X[:, perm[order[c]]] and, if partners, out[:, nev + c] = J conj(X[:, perm[order[c]]]) (FP64).
+cudaError_t launch_gather_pairs(const void* X, const int* perm, int64_t n, const int* order, int nev, int partners,
+                                void* out, cudaStream_t s);
+// out (FP64, 2n x kk real view) = V Z for the fixed-point basis, in exact integer sums (ritz.cu).
+cudaError_t launch_rotate_fx(const void* V, const int* vexp, int64_t n, int m, const double* Z, int kk, void* out,
+                             cudaStream_t s);
 
 // Mixed forms: the same Gram-Schmidt sequence in compensated FP32 ("double-float") arithmetic on a
 // basis stored as float4 {hi.re, hi.im, lo.re, lo.im} (gsdf.cu); y, alpha, beta and norms in FP64.
@@ -167,15 +188,11 @@ cudaError_t launch_ritz_jacobi(const double* T, int ldt, int m, int which, doubl
 // Vout[:, 0:kk] = V[:, 0:m] * Z[:, 0:kk] (V complex n x m, ld n; Z real m x kk, ld m).
 template <typename R>
 cudaError_t launch_rotate(const void* V, int64_t n, int m, const double* Z, int kk, void* Vout,
-                          cudaStream_t s);
+                          cudaStream_t s);   // the FP32 basis
 // V[:, c] = Vsrc[:, perm[c]] for c < k and V[:, k] = V[:, m] (restart shrink, Algorithm 1).
 template <typename R>
 cudaError_t launch_shrink(void* V, const void* Vsrc, int64_t n, const int* perm, int k, int m,
                           cudaStream_t s);
-// out[:, c] = V[:, order[c]] and, if partners, out[:, nev + c] = J conj(V[:, order[c]]).
-template <typename R>
-cudaError_t launch_gather_pairs(const void* V, int64_t n, const int* order, int nev, int partners,
-                                void* out, cudaStream_t s);
 // Column sums of squares partials -> sqrt into out[c] (c < ncol), partials [ncol][nblk].
 cudaError_t launch_reduce_norms(const double* part, int nblk, int ncol, double* out, cudaStream_t s);
 // Lemma 1 check partials: sum (v1 y2 - v2 y1), ||y||^2, ||v||^2 over all rows -> out[4].
@@ -263,6 +280,8 @@ cudaError_t gs_coop_occupancy(int m, int* per_sm);
 template <typename R>
 cudaError_t launch_gs_step_coop(const GSArgs& a, const double2* alpha_part, int n_alpha_part, int passes,
                                 double* nrm2, int grid, cudaStream_t s);
+template <> cudaError_t gs_coop_occupancy<double>(int, int*);
+template <> cudaError_t launch_gs_step_coop<double>(const GSArgs&, const double2*, int, int, double*, int, cudaStream_t);
 
 // The compensated-FP32 Gram-Schmidt of one Lanczos step as one cooperative launch (gsdf.cu); its
 // shared memory, so its occupancy, depends on rows_per_block and m of `a`.

@@ -1,6 +1,7 @@
 // ritz.cu -- the restart of Algorithm 1 on the device: Rayleigh-Ritz solve of T_m, the basis
 // rotation V_m := V_m Z_m (Corollary 2 keeps V and W = J V^* orthogonal under it), the shrink to
 // k + 1 vectors with v_{k+1} = v_{m+1}, and the output gather with partners y = J x^* (eq. (2)).
+#include "fixed.cuh"
 #include "internal.h"
 #include "ritz_dev.cuh"
 #include "../../include/jtrlan.h"
@@ -179,55 +180,108 @@ ritz_check_kernel(const double* __restrict__ T, int ldt, int m, int k, int kk, i
 }
 
 // ------------------------------------------------------------------ rotation V_m Z
-// Real GEMM on the interleaved view: V as a (2n x m) real matrix (column-major, ld 2n) times
-// Z (m x kk) gives Vout (2n x kk).  FP64: a 64 x 32 output tile per block, 8 outputs per thread.
-template <typename R>
-__global__ void __launch_bounds__(256)
-rotate_kernel(const R* __restrict__ V, int64_t rows, int m, const double* __restrict__ Z, int kk, R* __restrict__ out) {
-  constexpr int BM = 64, BN = 32, BK = 16;
-  __shared__ R As[BK][BM];
-  __shared__ double Bs[BK][BN];
-  const int tid = threadIdx.x;
-  const int64_t row0 = (int64_t)blockIdx.x * BM;
-  const int col0 = blockIdx.y * BN;
-  const int tr = tid % 16, tc = tid / 16;  // 4 rows (tr, tr+16, ...) x 2 cols (tc, tc+16)
-  double acc[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-  for (int k0 = 0; k0 < m; k0 += BK) {
-    for (int e = tid; e < BK * BM; e += 256) {
-      const int kk_ = e / BM, r = e % BM;
-      const int64_t gr = row0 + r;
-      As[kk_][r] = (gr < rows && k0 + kk_ < m) ? V[(int64_t)(k0 + kk_) * rows + gr] : (R)0;
-    }
-    for (int e = tid; e < BK * BN; e += 256) {
-      const int kk_ = e / BN, c = e % BN;
-      Bs[kk_][c] = (k0 + kk_ < m && col0 + c < kk) ? Z[(int64_t)(col0 + c) * m + k0 + kk_] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int x = 0; x < BK; ++x) {
-      double a[4], b[2];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = (double)As[x][tr + 16 * i];
-      b[0] = Bs[x][tc];
-      b[1] = Bs[x][tc + 16];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[i][0] = fma(a[i], b[0], acc[i][0]);
-        acc[i][1] = fma(a[i], b[1], acc[i][1]);
+// out (n x kk complex) = V Z for the fixed-point basis (fixed.cuh), Z real: exact integer sums of two-limb
+// products, 16 a clock and SM against 2 FP64 multiply-adds.  A lane owns a complex row and four columns
+// of Z (8 sums); the warps of a block share the row's loads through L1 and take other columns.  Z, scaled
+// by the columns' 2^e and converted on the scale of its largest entry per column, passes through shared
+// memory 64 rows at a time, the number of products a sum holds; then the sums leave for FP64.
+// A column of Z that is a unit vector (a locked pair's) copies that column of V to the last bit.
+// 8^4 (m 60): 58 us a launch, 199 us in FP64.
+constexpr int kRotK = 64, kRotC = 4, kRotGroups = 8;
+
+__global__ void __launch_bounds__(32 * kRotGroups)
+rotate_fx_kernel(const fxc* __restrict__ V, const int* __restrict__ vexp, int64_t n, int m, const double* __restrict__ Z,
+                 int kk, double2* __restrict__ out) {
+  __shared__ __align__(16) int2 zs[kRotK][kRotC * kRotGroups];
+  __shared__ int zk[kRotC * kRotGroups], zunit[kRotC * kRotGroups];   // K; k (or ~k for -1) of a unit column, else m
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, cols = kRotC * (blockDim.x >> 5);
+  const int c0 = blockIdx.y * cols;
+  const int64_t p = (int64_t)blockIdx.x * 32 + lane;
+  for (int c = w; c < cols; c += blockDim.x >> 5) {     // K of each scaled column of Z
+    int f = 0, cnt = 0, unit = m;
+    if (c0 + c < kk)
+      for (int k = lane; k < m; k += 32) {
+        const double z = Z[(int64_t)(c0 + c) * m + k];
+        const int g = fx_field(z);
+        f = max(f, g ? max(g + vexp[k] - 1023, 1) : 0);
+        if (g >= 1023 - 60) {
+          ++cnt;
+          unit = __double2hiint(z) < 0 ? ~k : k;
+        }
       }
+    f = __reduce_max_sync(0xffffffffu, f);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    const unsigned has = __ballot_sync(0xffffffffu, unit != m);
+    if (has) unit = __shfl_sync(0xffffffffu, unit, __ffs(has) - 1);
+    if (lane == 0) {
+      zk[c] = f + 1;
+      zunit[c] = cnt == 1 ? unit : m;
+    }
+  }
+  double2 o[kRotC];
+#pragma unroll
+  for (int c = 0; c < kRotC; ++c) o[c] = make_double2(0.0, 0.0);
+  for (int k0 = 0; k0 < m; k0 += kRotK) {
+    const int kn = min(kRotK, m - k0);
+    __syncthreads();
+    for (int e = threadIdx.x; e < cols * kRotK; e += blockDim.x) {
+      const int k = e % kRotK, c = e / kRotK;
+      int2 v = make_int2(0, 0);
+      if (k < kn && c0 + c < kk) {
+        const fx2 t = fx_limbs<true>(Z[(int64_t)(c0 + c) * m + k0 + k], zk[c] - (vexp[k0 + k] - 1023));
+        v = make_int2(t.h, t.l);
+      }
+      zs[k][c] = v;
     }
     __syncthreads();
-  }
+    FxAcc a[kRotC][2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t gr = row0 + tr + 16 * i;
-    if (gr >= rows) continue;
+    for (int c = 0; c < kRotC; ++c) {
+      fx_zero(a[c][0]);
+      fx_zero(a[c][1]);
+    }
+    if (p < n) {
+      const fxc* v = V + (int64_t)k0 * n + p;
+      auto mac = [&](fxc x, int k) {
+        const fx2 re = fx_round(x.re), im = fx_round(x.im);
 #pragma unroll
-    for (int jx = 0; jx < 2; ++jx) {
-      const int gc = col0 + tc + 16 * jx;
-      if (gc < kk) out[(int64_t)gc * rows + gr] = (R)acc[i][jx];
+        for (int c = 0; c < kRotC; c += 2) {
+          const int4 z = *reinterpret_cast<const int4*>(&zs[k][kRotC * w + c]);
+          fx_mac(a[c][0], re, fx2{z.x, z.y});
+          fx_mac(a[c][1], im, fx2{z.x, z.y});
+          fx_mac(a[c + 1][0], re, fx2{z.z, z.w});
+          fx_mac(a[c + 1][1], im, fx2{z.z, z.w});
+        }
+      };
+      int k = 0;
+      for (; k + 3 < kn; k += 4) {
+        fxc x[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) x[t] = v[(int64_t)(k + t) * n];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) mac(x[t], k + t);
+      }
+      for (; k < kn; ++k) mac(v[(int64_t)k * n], k);
+    }
+#pragma unroll
+    for (int c = 0; c < kRotC; ++c) {
+      const int K = zk[kRotC * w + c];
+      const double re = fx_lane_value(a[c][0], K), im = fx_lane_value(a[c][1], K);
+      if (k0 == 0) o[c] = make_double2(re, im);
+      else o[c] = make_double2(o[c].x + re, o[c].y + im);
     }
   }
+  if (p < n)
+#pragma unroll
+    for (int c = 0; c < kRotC; ++c) {
+      const int u = zunit[kRotC * w + c], k = u < 0 ? ~u : u;
+      if (k < m) {
+        const fxc x = V[(int64_t)k * n + p];
+        const double re = fx_load(x.re, vexp[k]), im = fx_load(x.im, vexp[k]);
+        o[c] = u < 0 ? make_double2(-re, -im) : make_double2(re, im);
+      }
+      if (c0 + kRotC * w + c < kk) out[(int64_t)(c0 + kRotC * w + c) * n + p] = o[c];
+    }
 }
 
 // FP32 rotation for the mixed-precision phase: Z rounded to FP32, FP32 accumulation.
@@ -286,25 +340,6 @@ __global__ void shrink_kernel(cplx<R>* V, const cplx<R>* Vsrc, int64_t n, const 
   cplx<R>* dst = V + (int64_t)c * n;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     dst[i] = src[i];
-}
-
-template <typename R>
-__global__ void gather_pairs_kernel(const cplx<R>* V, int64_t n, const int* order, int nev, int partners,
-                                    cplx<R>* out) {
-  const int c = blockIdx.y;
-  const int64_t h = n / 2;
-  const cplx<R>* src = V + (int64_t)order[c] * n;
-  cplx<R>* dst = out + (int64_t)c * n;
-  cplx<R>* dstp = out + (int64_t)(nev + c) * n;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < h; i += (int64_t)gridDim.x * blockDim.x) {
-    const cplx<R> x1 = src[i], x2 = src[h + i];
-    dst[i] = x1;
-    dst[h + i] = x2;
-    if (partners) {  // J x^* = [-x2^*; x1^*]
-      dstp[i] = mk<R>(-x2.x, x2.y);
-      dstp[h + i] = mk<R>(x1.x, -x1.y);
-    }
-  }
 }
 
 __global__ void reduce_norms_kernel(const double* part, int nblk, double* out) {
@@ -382,16 +417,21 @@ cudaError_t launch_ritz_jacobi(const double* T, int ldt, int m, int which, doubl
   return jacobi_launch(T, ldt, m, which, lam, Z, work, nullptr, nullptr, s);
 }
 
-template <typename R>
-cudaError_t launch_rotate(const void* V, int64_t n, int m, const double* Z, int kk, void* Vout, cudaStream_t s) {
+template <>
+cudaError_t launch_rotate<float>(const void* V, int64_t n, int m, const double* Z, int kk, void* Vout, cudaStream_t s) {
   const int64_t rows = 2 * n;
-  if constexpr (sizeof(R) == sizeof(float)) {
-    dim3 grid((unsigned)((rows + 127) / 128), (unsigned)((kk + 31) / 32));
-    rotate32_kernel<<<grid, 256, 0, s>>>((const float*)V, rows, m, Z, kk, (float*)Vout);
-    return cudaGetLastError();
-  }
-  dim3 grid((unsigned)((rows + 63) / 64), (unsigned)((kk + 31) / 32));
-  rotate_kernel<R><<<grid, 256, 0, s>>>((const R*)V, rows, m, Z, kk, (R*)Vout);
+  dim3 grid((unsigned)((rows + 127) / 128), (unsigned)((kk + 31) / 32));
+  rotate32_kernel<<<grid, 256, 0, s>>>((const float*)V, rows, m, Z, kk, (float*)Vout);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rotate_fx(const void* V, const int* vexp, int64_t n, int m, const double* Z, int kk, void* out,
+                             cudaStream_t s) {
+  const int need = (kk + kRotC - 1) / kRotC;                       // column groups
+  const int tiles = (need + kRotGroups - 1) / kRotGroups;
+  const int groups = (need + tiles - 1) / tiles;                   // a block's, evenly filled
+  rotate_fx_kernel<<<dim3((unsigned)((n + 31) / 32), (unsigned)tiles), 32 * groups, 0, s>>>(
+      (const fxc*)V, vexp, n, m, Z, kk, (double2*)out);
   return cudaGetLastError();
 }
 
@@ -399,14 +439,6 @@ template <typename R>
 cudaError_t launch_shrink(void* V, const void* Vsrc, int64_t n, const int* perm, int k, int m, cudaStream_t s) {
   dim3 grid(grid_for(n) / 4 + 1, k + 1);
   shrink_kernel<R><<<grid, 256, 0, s>>>((cplx<R>*)V, (const cplx<R>*)Vsrc, n, perm, k, m);
-  return cudaGetLastError();
-}
-
-template <typename R>
-cudaError_t launch_gather_pairs(const void* V, int64_t n, const int* order, int nev, int partners, void* out,
-                                cudaStream_t s) {
-  dim3 grid(grid_for(n / 2) / 4 + 1, nev);
-  gather_pairs_kernel<R><<<grid, 256, 0, s>>>((const cplx<R>*)V, n, order, nev, partners, (cplx<R>*)out);
   return cudaGetLastError();
 }
 
@@ -422,10 +454,6 @@ cudaError_t launch_report(const double* lam, const double* Z, int m, const doubl
   return cudaGetLastError();
 }
 
-template cudaError_t launch_rotate<double>(const void*, int64_t, int, const double*, int, void*, cudaStream_t);
-template cudaError_t launch_rotate<float>(const void*, int64_t, int, const double*, int, void*, cudaStream_t);
 template cudaError_t launch_shrink<float>(void*, const void*, int64_t, const int*, int, int, cudaStream_t);
-template cudaError_t launch_shrink<double>(void*, const void*, int64_t, const int*, int, int, cudaStream_t);
-template cudaError_t launch_gather_pairs<double>(const void*, int64_t, const int*, int, int, void*, cudaStream_t);
 
 }  // namespace jtr
