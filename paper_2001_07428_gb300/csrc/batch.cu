@@ -16,6 +16,7 @@
 // passes <= gs_passes, Jacobi sweeps <= 40).
 #include <math.h>
 
+#include "fixed.cuh"
 #include "internal.h"
 #include "ritz_dev.cuh"
 #include "../../include/jtrlan.h"
@@ -115,6 +116,18 @@ struct Shared {
   int ok, status, icnv, k, nlocked, inst;
   double tmax;
 };
+// The integer form's small state, in the place of coef4: K of the columns of V and of Z, unit columns of Z.
+struct FxState {
+  int vexp[kMaxM + 1], zk[kMaxM], zunit[kMaxM], misc[4], imax[16];
+};
+static_assert(sizeof(FxState) <= sizeof(Shared::coef4), "FxState lies in coef4");
+// The update's coefficients, in the Ritz solve's scratch (zb): small columns, limbs of the large ones, their list.
+struct FxCoef {
+  int4* sm;
+  int4* lg;
+  int* list;
+};
+static_assert((3 * sizeof(int4) + sizeof(int)) * 2 <= 2 * 32 * sizeof(double), "52 (m + 1) <= 104 m <= 512 m bytes");
 
 __host__ __device__ inline size_t up16(size_t b) { return (b + 15) & ~(size_t)15; }
 
@@ -282,69 +295,10 @@ __device__ void cta_matvec_df1(const float4* A11, const float4* A12, int64_t h, 
   }
 }
 
-template <bool DF, int MVR>
-__device__ void cta_matvec(const BatchArgs& a, int64_t h, int64_t off, const double2* x, const float4* x4, double2* y,
-                           double* red) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if constexpr (DF) {
-    if constexpr (MVR == 1)
-      cta_matvec_df1((const float4*)a.A11 + off, (const float4*)a.A12 + off, h, x4, y);
-    else
-      cta_matvec_df((const float4*)a.A11 + off, (const float4*)a.A12 + off, h, x4, y);
-  } else if constexpr (MVR == 2) {   // two rows per warp (r and r + nw) sharing the loads of x
-    for (int64_t r = w; r < h; r += 2 * nw) {
-      const int64_t r2 = r + nw;
-      const bool two = r2 < h;
-      const double2* r11 = (const double2*)a.A11 + off + r * h;
-      const double2* r12 = (const double2*)a.A12 + off + r * h;
-      const double2* s11 = (const double2*)a.A11 + off + (two ? r2 : r) * h;
-      const double2* s12 = (const double2*)a.A12 + off + (two ? r2 : r) * h;
-      double2 y1 = make_double2(0, 0), y2 = make_double2(0, 0), z1 = make_double2(0, 0), z2 = make_double2(0, 0);
-      for (int64_t c = lane; c < h; c += 32) {
-        const double2 x1 = x[c], x2 = x[h + c];
-        const double2 a11 = r11[c], a12 = r12[c];
-        y1 = cfma(a11, x1, y1);
-        y1 = cfma(a12, x2, y1);
-        y2 = cfmac(a11, x2, y2);
-        y2 = cfmac(make_double2(-a12.x, -a12.y), x1, y2);
-        if (two) {
-          const double2 b11 = s11[c], b12 = s12[c];
-          z1 = cfma(b11, x1, z1);
-          z1 = cfma(b12, x2, z1);
-          z2 = cfmac(b11, x2, z2);
-          z2 = cfmac(make_double2(-b12.x, -b12.y), x1, z2);
-        }
-      }
-      const double v0 = warp_sum(y1.x), v1 = warp_sum(y1.y), v2 = warp_sum(y2.x), v3 = warp_sum(y2.y);
-      const double u0 = warp_sum(z1.x), u1 = warp_sum(z1.y), u2 = warp_sum(z2.x), u3 = warp_sum(z2.y);
-      if (lane == 0) {
-        y[r] = make_double2(v0, v1);
-        y[h + r] = make_double2(v2, v3);
-        if (two) {
-          y[r2] = make_double2(u0, u1);
-          y[h + r2] = make_double2(u2, u3);
-        }
-      }
-    }
-  } else {
-    for (int64_t r = w; r < h; r += nw) {
-      const double2* r11 = (const double2*)a.A11 + off + r * h;
-      const double2* r12 = (const double2*)a.A12 + off + r * h;
-      double2 y1 = make_double2(0, 0), y2 = make_double2(0, 0);
-      for (int64_t c = lane; c < h; c += 32) {
-        const double2 a11 = r11[c], a12 = r12[c], x1 = x[c], x2 = x[h + c];
-        y1 = cfma(a11, x1, y1);
-        y1 = cfma(a12, x2, y1);
-        y2 = cfmac(a11, x2, y2);
-        y2 = cfmac(make_double2(-a12.x, -a12.y), x1, y2);
-      }
-      const double v0 = warp_sum(y1.x), v1 = warp_sum(y1.y), v2 = warp_sum(y2.x), v3 = warp_sum(y2.y);
-      if (lane == 0) {
-        y[r] = make_double2(v0, v1);
-        y[h + r] = make_double2(v2, v3);
-      }
-    }
-  }
+template <int MVR>
+__device__ void cta_matvec(const BatchArgs& a, int64_t h, int64_t off, const float4* x4, double2* y) {
+  if constexpr (MVR == 1) cta_matvec_df1((const float4*)a.A11 + off, (const float4*)a.A12 + off, h, x4, y);
+  else cta_matvec_df((const float4*)a.A11 + off, (const float4*)a.A12 + off, h, x4, y);
   __syncthreads();
 }
 
@@ -353,222 +307,533 @@ __device__ void cta_matvec(const BatchArgs& a, int64_t h, int64_t off, const dou
 // coefficients in coef4 (c_v of column i at 2i, c_w at 2i + 1), so no FP64 work is left per element.
 // The double-float form walks (column, 32-row chunk) pairs with the next chunk's loads issued before
 // the current chunk's arithmetic and reduces the 4 sums of a column with one reduce-scatter.
-template <bool DF>
-__device__ void cta_dot(const void* Vv, int64_t n, int64_t h, int j, const double2* y, float4* y4, double* coef,
+__device__ void cta_dot(const float4* V, int64_t n, int64_t h, int j, const double2* y, float4* y4, double* coef,
                         float4* coef4) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if constexpr (DF) {
-    for (int64_t p = threadIdx.x; p < n; p += blockDim.x) y4[p] = b_split(y[p]);
-    __syncthreads();
-    const float4* V = (const float4*)Vv;
-    const int C = (int)((h + 31) >> 5);
-    const int ncol = (w <= j) ? (j - w) / nw + 1 : 0;
-    const int total = ncol * C;
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto fetch = [&](int t, int u, float4& v1, float4& v2) {
-      const int64_t p = lane + 32 * u;
-      const int64_t i = w + (int64_t)t * nw;
-      v1 = v2 = z4;
-      if (p < h) {
-        v1 = V[i * n + p];
-        v2 = V[i * n + h + p];
-      }
-    };
-    float4 c1, c2;
-    if (total > 0) fetch(0, 0, c1, c2);
-    float sv[4] = {0.f, 0.f, 0.f, 0.f}, ev[4] = {0.f, 0.f, 0.f, 0.f};   // c_v re, im, c_w re, im
-    int t = 0, u = 0;
-    for (int it = 0; it < total; ++it) {
-      int tn = t, un = u + 1;
-      if (un == C) {
-        un = 0;
-        ++tn;
-      }
-      float4 n1 = z4, n2 = z4;
-      if (it + 1 < total) fetch(tn, un, n1, n2);
-      const int64_t p = lane + 32 * u;
-      if (p < h) {
-        const float4 y1 = y4[p], y2 = y4[h + p];
-        b_caccc(&sv[0], &ev[0], c1, y1);       // c_v = sum conj(v1) y1 + conj(v2) y2
-        b_caccc(&sv[0], &ev[0], c2, y2);
-        b_cacc(&sv[2], &ev[2], c1, y2);        // c_w = sum v1 y2 - v2 y1
-        b_cacc(&sv[2], &ev[2], c2, y1, -1.f);
-      }
-      if (u == C - 1) {
-        const double v = df_reduce4(sv, ev);
-        const int i = w + t * nw;
-        if ((lane & 7) == 0) coef[4 * i + (lane >> 3)] = v;
+  for (int64_t p = threadIdx.x; p < n; p += blockDim.x) y4[p] = b_split(y[p]);
+  __syncthreads();
+  const int C = (int)((h + 31) >> 5);
+  const int ncol = (w <= j) ? (j - w) / nw + 1 : 0;
+  const int total = ncol * C;
+  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto fetch = [&](int t, int u, float4& v1, float4& v2) {
+    const int64_t p = lane + 32 * u;
+    const int64_t i = w + (int64_t)t * nw;
+    v1 = v2 = z4;
+    if (p < h) {
+      v1 = V[i * n + p];
+      v2 = V[i * n + h + p];
+    }
+  };
+  float4 c1, c2;
+  if (total > 0) fetch(0, 0, c1, c2);
+  float sv[4] = {0.f, 0.f, 0.f, 0.f}, ev[4] = {0.f, 0.f, 0.f, 0.f};   // c_v re, im, c_w re, im
+  int t = 0, u = 0;
+  for (int it = 0; it < total; ++it) {
+    int tn = t, un = u + 1;
+    if (un == C) {
+      un = 0;
+      ++tn;
+    }
+    float4 n1 = z4, n2 = z4;
+    if (it + 1 < total) fetch(tn, un, n1, n2);
+    const int64_t p = lane + 32 * u;
+    if (p < h) {
+      const float4 y1 = y4[p], y2 = y4[h + p];
+      b_caccc(&sv[0], &ev[0], c1, y1);       // c_v = sum conj(v1) y1 + conj(v2) y2
+      b_caccc(&sv[0], &ev[0], c2, y2);
+      b_cacc(&sv[2], &ev[2], c1, y2);        // c_w = sum v1 y2 - v2 y1
+      b_cacc(&sv[2], &ev[2], c2, y1, -1.f);
+    }
+    if (u == C - 1) {
+      const double v = df_reduce4(sv, ev);
+      const int i = w + t * nw;
+      if ((lane & 7) == 0) coef[4 * i + (lane >> 3)] = v;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) sv[k] = ev[k] = 0.f;
+      for (int k = 0; k < 4; ++k) sv[k] = ev[k] = 0.f;
+    }
+    c1 = n1;
+    c2 = n2;
+    t = tn;
+    u = un;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+    coef4[2 * i] = b_split(make_double2(coef[4 * i], coef[4 * i + 1]));
+    coef4[2 * i + 1] = b_split(make_double2(coef[4 * i + 2], coef[4 * i + 3]));
+  }
+  __syncthreads();
+}
+
+// y -= V c_v + W c_w; returns ||y||^2 (block-wide): the CTA's threads form G = blockDim / hp groups of hp >= h threads (h rounded up to 32); group g
+// takes columns g, g + G, ... for every row pair, with the next column's loads issued before the
+// current one's arithmetic; groups 1 .. G-1 leave their compensated partial sums in `part`
+// (8 floats per thread) and group 0 adds them and updates y.
+__device__ double cta_update(const float4* V, int64_t n, int64_t h, int j, const float4* coef4, double2* y, float* part,
+                             double* red, int gs_groups) {
+  double nrm = 0.0;
+  // compensated sums of V c_v + W c_w over columns g0, g0 + G, ... <= j for row pair p
+  auto accumulate = [&](int64_t p, int g0, int G, float* s, float* e) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = e[k] = 0.f;
+    if (g0 > j) return;
+    float4 v1 = V[(int64_t)g0 * n + p], v2 = V[(int64_t)g0 * n + h + p];
+    for (int i = g0; i <= j; i += G) {
+      float4 n1 = v1, n2 = v2;
+      if (i + G <= j) {
+        n1 = V[(int64_t)(i + G) * n + p];
+        n2 = V[(int64_t)(i + G) * n + h + p];
       }
-      c1 = n1;
-      c2 = n2;
-      t = tn;
-      u = un;
+      const float4 cv = coef4[2 * i], cw = coef4[2 * i + 1];
+      b_cacc(&s[0], &e[0], v1, cv);          // (V c_v + W c_w)_1 = v1 c_v - conj(v2) c_w
+      b_caccc(&s[0], &e[0], v2, cw, -1.f);
+      b_cacc(&s[2], &e[2], v2, cv);          // (V c_v + W c_w)_2 = v2 c_v + conj(v1) c_w
+      b_caccc(&s[2], &e[2], v1, cw);
+      v1 = n1;
+      v2 = n2;
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-      coef4[2 * i] = b_split(make_double2(coef[4 * i], coef[4 * i + 1]));
-      coef4[2 * i + 1] = b_split(make_double2(coef[4 * i + 2], coef[4 * i + 3]));
+  };
+  auto apply = [&](int64_t p, const float* s, const float* e) {
+    double2 y1 = y[p], y2 = y[h + p];
+    y1.x -= (double)s[0] + (double)e[0];
+    y1.y -= (double)s[1] + (double)e[1];
+    y2.x -= (double)s[2] + (double)e[2];
+    y2.y -= (double)s[3] + (double)e[3];
+    y[p] = y1;
+    y[h + p] = y2;
+    nrm += cabs2(y1) + cabs2(y2);
+  };
+  const int hp = (int)(((h + 31) >> 5) << 5);
+  float s[4], e[4];
+  if (hp <= (int)blockDim.x) {               // one sweep: G groups of hp threads
+    int G = (int)blockDim.x / hp;
+    if (gs_groups > 0 && G > gs_groups) G = gs_groups;   // tile shape: fewer, longer column walks
+    const int g = (int)threadIdx.x / hp, tl = (int)threadIdx.x - g * hp;
+    const bool active = g < G && tl < h;
+    if (active) accumulate(tl, g, G, s, e);
+    if (G > 1) {
+      if (active && g > 0) {
+        float* pp = part + (size_t)8 * ((g - 1) * hp + tl);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          pp[k] = s[k];
+          pp[4 + k] = e[k];
+        }
+      }
+      __syncthreads();
+      if (active && g == 0)
+        for (int gg = 1; gg < G; ++gg) {
+          const float* pp = part + (size_t)8 * ((gg - 1) * hp + tl);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) df_add(s[k], e[k], pp[k], pp[4 + k]);
+        }
     }
+    if (active && g == 0) apply(tl, s, e);
   } else {
-    for (int i = w; i <= j; i += nw) {
-      const double2* vi = (const double2*)Vv + (int64_t)i * n;
-      double2 cv = make_double2(0, 0), cw = make_double2(0, 0);
-      for (int64_t p = lane; p < h; p += 32) {
-        const double2 v1 = vi[p], v2 = vi[h + p], y1 = y[p], y2 = y[h + p];
-        cv = cfmac(v1, y1, cv);
-        cv = cfmac(v2, y2, cv);
-        cw = cfma(v1, y2, cw);
-        cw = cfma(make_double2(-v2.x, -v2.y), y1, cw);
+    for (int64_t p = threadIdx.x; p < h; p += blockDim.x) {
+      accumulate(p, 0, 1, s, e);
+      apply(p, s, e);
+    }
+  }
+  return blk_sum(nrm, red);
+}
+
+// Vt[:, c] = V Z[:, c] for c in [c0, c1), rows 2n real (FP64 target); Z as (hi, lo) float pairs.
+__device__ void cta_rotate(const float4* V, int64_t n, int m, const float2* Zf, int c0, int c1, double2* Vt) {
+  for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
+    for (int cb = c0; cb < c1; cb += 4) {
+      float sr[4] = {0, 0, 0, 0}, er[4] = {0, 0, 0, 0}, si[4] = {0, 0, 0, 0}, ei[4] = {0, 0, 0, 0};
+      for (int i = 0; i < m; ++i) {
+        const float4 v = V[(int64_t)i * n + p];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (cb + q < c1) {
+            const float2 z = Zf[(size_t)(cb + q) * m + i];
+            b_df_acc(sr[q], er[q], v.x, v.z, z.x, z.y);
+            b_df_acc(si[q], ei[q], v.y, v.w, z.x, z.y);
+          }
+        }
       }
-      const double c0 = warp_sum(cv.x), c1 = warp_sum(cv.y), c2 = warp_sum(cw.x), c3 = warp_sum(cw.y);
-      if (lane == 0) {
-        coef[4 * i] = c0;
-        coef[4 * i + 1] = c1;
-        coef[4 * i + 2] = c2;
-        coef[4 * i + 3] = c3;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (cb + q < c1)
+          Vt[(int64_t)(cb + q) * n + p] = make_double2((double)sr[q] + (double)er[q], (double)si[q] + (double)ei[q]);
+    }
+  }
+  __syncthreads();
+}
+
+// ------------------------------------------------------------------ the integer form of FP64
+// Plain FP64 in this kernel was bound by the FP64 pipe (the products at 45% of it, two thirds of the
+// time).  Here A and the basis are 60-bit fixed point (fixed.cuh; one exponent per instance and per
+// column) and the products, the inner products, the update and the rotation are exact integer sums.
+
+// Largest int over the block (every thread gets it).
+__device__ __forceinline__ int blk_imax(int v, int* buf) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  const int nw = blockDim.x >> 5;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = v;
+  __syncthreads();
+  for (int i = 0; i < nw; ++i) v = max(v, buf[i]);
+  return v;
+}
+// blk_sum with the warps' sums in integers: five FP64 adds a warp hold their quarter of the SM for 320 clocks.
+__device__ __forceinline__ double blk_isum(double v, double* red) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  v = fx_warp_total(v);
+  __syncthreads();
+  if (lane == 0) red[w] = v;
+  __syncthreads();
+  if (w == 0) {
+    double t = lane < nw ? red[lane] : 0.0;
+    for (int o = 1; o < nw; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) red[32] = t;
+  }
+  __syncthreads();
+  return red[32];
+}
+
+// Products of one pair (a11, a12) with (x1, x2) into the seven sums
+// Re y1 = s0 - s1, Im y1 = s2, Re y2 = s3 - s4, Im y2 = s5 - s6.
+__device__ __forceinline__ void mv_pair(FxAcc* s, fxc a11, fxc a12, int4 x1, int4 x2) {
+  const fx2 p{x1.x, x1.y}, q{x1.z, x1.w}, r{x2.x, x2.y}, t{x2.z, x2.w};
+  const fx2 a = fx_round(a11.re), b = fx_round(a11.im), c = fx_round(a12.re), d = fx_round(a12.im);
+  fx_mac(s[0], a, p); fx_mac(s[0], c, r); fx_mac(s[1], b, q); fx_mac(s[1], d, t);
+  fx_mac(s[2], a, q); fx_mac(s[2], b, p); fx_mac(s[2], c, t); fx_mac(s[2], d, r);
+  fx_mac(s[3], a, r); fx_mac(s[3], b, t); fx_mac(s[4], c, p); fx_mac(s[4], d, q);
+  fx_mac(s[5], a, t); fx_mac(s[5], d, p); fx_mac(s[6], b, r); fx_mac(s[6], c, q);
+}
+
+// y = A x: a warp a row, the lanes its columns; xl holds x as limbs on K = Kx, A is on Ka (2048: an entry
+// of A is infinite or NaN, and so is y).  Up to 512 columns a sum holds (64 products); the sums of eight
+// rows are kept one a lane and leave for FP64 together.
+__device__ void cta_matvec_fx(const fxc* A11, const fxc* A12, int64_t h, const int4* xl, int Kx, int Ka, double2* y) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int64_t c0 = 0; c0 < h; c0 += 512) {
+    const int ce = (int)min((int64_t)512, h - c0);
+    const int4* x1 = xl + c0;
+    const int4* x2 = xl + h + c0;
+    int4 keep = make_int4(0, 0, 0, 0);
+    int k = 0;
+    for (int64_t row = w; row < h; row += nw) {
+      const fxc* r11 = A11 + row * h + c0;
+      const fxc* r12 = A12 + row * h + c0;
+      FxAcc s[7];
+#pragma unroll
+      for (int t = 0; t < 7; ++t) fx_zero(s[t]);
+      int c = lane;
+#pragma unroll 1
+      for (; c + 32 < ce; c += 64) {
+        const fxc a0 = r11[c], b0 = r12[c], a1 = r11[c + 32], b1 = r12[c + 32];
+        mv_pair(s, a0, b0, x1[c], x2[c]);
+        mv_pair(s, a1, b1, x1[c + 32], x2[c + 32]);
+      }
+      if (c < ce) mv_pair(s, r11[c], r12[c], x1[c], x2[c]);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int4 p = fx_warp_sum(t == 0 ? fx_diff(s[0], s[1]) : t == 1 ? s[2] : fx_diff(s[2 * t - 1], s[2 * t]));
+        if (lane == 4 * k + t) keep = p;
+      }
+      if (++k == 8 || row + nw >= h) {
+        const int64_t rl = row - (int64_t)nw * (k - 1 - (lane >> 2));   // this lane's row
+        if ((lane >> 2) < k) {
+          double* out = (double*)y + ((lane & 2) ? 2 * (h + rl) : 2 * rl) + (lane & 1);
+          const double v = Ka >= 2048 ? (double)NAN : fx_value(keep, Ka, Kx);
+          *out = c0 == 0 ? v : *out + v;
+        }
+        k = 0;
       }
     }
   }
   __syncthreads();
 }
 
-// y -= V c_v + W c_w; returns ||y||^2 (block-wide).  FP64: each thread a row pair.  Double-float:
-// the CTA's threads form G = blockDim / hp groups of hp >= h threads (h rounded up to 32); group g
-// takes columns g, g + G, ... for every row pair, with the next column's loads issued before the
-// current one's arithmetic; groups 1 .. G-1 leave their compensated partial sums in `part`
-// (8 floats per thread) and group 0 adds them and updates y.
-template <bool DF>
-__device__ double cta_update(const void* Vv, int64_t n, int64_t h, int j, const double* coef, const float4* coef4,
-                             double2* y, float* part, double* red, int gs_groups) {
-  double nrm = 0.0;
-  if constexpr (DF) {
-    const float4* V = (const float4*)Vv;
-    // compensated sums of V c_v + W c_w over columns g0, g0 + G, ... <= j for row pair p
-    auto accumulate = [&](int64_t p, int g0, int G, float* s, float* e) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) s[k] = e[k] = 0.f;
-      if (g0 > j) return;
-      float4 v1 = V[(int64_t)g0 * n + p], v2 = V[(int64_t)g0 * n + h + p];
-      for (int i = g0; i <= j; i += G) {
-        float4 n1 = v1, n2 = v2;
-        if (i + G <= j) {
-          n1 = V[(int64_t)(i + G) * n + p];
-          n2 = V[(int64_t)(i + G) * n + h + p];
-        }
-        const float4 cv = coef4[2 * i], cw = coef4[2 * i + 1];
-        b_cacc(&s[0], &e[0], v1, cv);          // (V c_v + W c_w)_1 = v1 c_v - conj(v2) c_w
-        b_caccc(&s[0], &e[0], v2, cw, -1.f);
-        b_cacc(&s[2], &e[2], v2, cv);          // (V c_v + W c_w)_2 = v2 c_v + conj(v1) c_w
-        b_caccc(&s[2], &e[2], v1, cw);
-        v1 = n1;
-        v2 = n2;
-      }
-    };
-    auto apply = [&](int64_t p, const float* s, const float* e) {
-      double2 y1 = y[p], y2 = y[h + p];
-      y1.x -= (double)s[0] + (double)e[0];
-      y1.y -= (double)s[1] + (double)e[1];
-      y2.x -= (double)s[2] + (double)e[2];
-      y2.y -= (double)s[3] + (double)e[3];
-      y[p] = y1;
-      y[h + p] = y2;
-      nrm += cabs2(y1) + cabs2(y2);
-    };
-    const int hp = (int)(((h + 31) >> 5) << 5);
-    float s[4], e[4];
-    if (hp <= (int)blockDim.x) {               // one sweep: G groups of hp threads
-      int G = (int)blockDim.x / hp;
-      if (gs_groups > 0 && G > gs_groups) G = gs_groups;   // tile shape: fewer, longer column walks
-      const int g = (int)threadIdx.x / hp, tl = (int)threadIdx.x - g * hp;
-      const bool active = g < G && tl < h;
-      if (active) accumulate(tl, g, G, s, e);
-      if (G > 1) {
-        if (active && g > 0) {
-          float* pp = part + (size_t)8 * ((g - 1) * hp + tl);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            pp[k] = s[k];
-            pp[4 + k] = e[k];
-          }
-        }
-        __syncthreads();
-        if (active && g == 0)
-          for (int gg = 1; gg < G; ++gg) {
-            const float* pp = part + (size_t)8 * ((gg - 1) * hp + tl);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) df_add(s[k], e[k], pp[k], pp[4 + k]);
-          }
-      }
-      if (active && g == 0) apply(tl, s, e);
-    } else {
-      for (int64_t p = threadIdx.x; p < h; p += blockDim.x) {
-        accumulate(p, 0, 1, s, e);
-        apply(p, s, e);
-      }
-    }
-  } else {
-    for (int64_t p = threadIdx.x; p < h; p += blockDim.x) {
-      double2 y1 = y[p], y2 = y[h + p];
-      const double2* V = (const double2*)Vv;
-      double2 a1 = make_double2(0, 0), a2 = make_double2(0, 0);
-      for (int i = 0; i <= j; ++i) {
-        const double2 v1 = V[(int64_t)i * n + p], v2 = V[(int64_t)i * n + h + p];
-        const double2 cv = make_double2(coef[4 * i], coef[4 * i + 1]), cw = make_double2(coef[4 * i + 2], coef[4 * i + 3]);
-        a1 = cfma(v1, cv, a1);
-        a1 = cfmac(v2, make_double2(-cw.x, -cw.y), a1);
-        a2 = cfma(v2, cv, a2);
-        a2 = cfmac(v1, cw, a2);
-      }
-      y1.x -= a1.x; y1.y -= a1.y; y2.x -= a2.x; y2.y -= a2.y;
-      y[p] = y1;
-      y[h + p] = y2;
-      nrm += cabs2(y1) + cabs2(y2);
-    }
+// Limbs of the FP64 vector y (n entries) into yl; returns their K.
+__device__ int cta_limbs(const double2* y, int64_t n, int4* yl, int* buf) {
+  int ex = 0;
+  for (int64_t p = threadIdx.x; p < n; p += blockDim.x) ex = max(ex, max(fx_field(y[p].x), fx_field(y[p].y)));
+  const int K = blk_imax(ex, buf) + 1;
+  for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
+    const fx2 re = fx_limbs<true>(y[p].x, K), im = fx_limbs<true>(y[p].y, K);
+    yl[p] = make_int4(re.h, re.l, im.h, im.l);
   }
-  return blk_sum(nrm, red);
+  __syncthreads();
+  return K;
 }
 
-// Vt[:, c] = V Z[:, c] for c in [c0, c1), rows 2n real (FP64 target); the double-float form reads
-// Z as (hi, lo) float pairs from Zf.
-template <bool DF>
-__device__ void cta_rotate(const void* Vv, int64_t n, int m, const double* Z, const float2* Zf, int c0, int c1,
-                           double2* Vt) {
-  for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
-    for (int cb = c0; cb < c1; cb += 4) {
-      double ar[4] = {0, 0, 0, 0}, ai[4] = {0, 0, 0, 0};
-      float sr[4] = {0, 0, 0, 0}, er[4] = {0, 0, 0, 0}, si[4] = {0, 0, 0, 0}, ei[4] = {0, 0, 0, 0};
-      for (int i = 0; i < m; ++i) {
-        if (!DF) {
-          const double2 v = ((const double2*)Vv)[(int64_t)i * n + p];
+// c_v = V^H y and c_w = W^H y for columns 0..j into coef: a warp a column, the lanes its row pairs.
+__device__ void cta_dot_fx(const fxc* V, const int* vexp, int64_t n, int64_t h, int j, const int4* yl, int Ky, double* coef) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  auto pair = [](FxAcc* s, fxc v1, fxc v2, int4 w1, int4 w2) {   // as dot_row of gsfx.cu
+    const fx2 y1x{w1.x, w1.y}, y1y{w1.z, w1.w}, y2x{w2.x, w2.y}, y2y{w2.z, w2.w};
+    const fx2 a = fx_round(v1.re), b = fx_round(v1.im), c = fx_round(v2.re), d = fx_round(v2.im);
+    fx_mac(s[0], a, y1x); fx_mac(s[0], b, y1y); fx_mac(s[0], c, y2x); fx_mac(s[0], d, y2y);
+    fx_mac(s[1], a, y1y); fx_mac(s[1], c, y2y); fx_mac(s[2], b, y1x); fx_mac(s[2], d, y2x);
+    fx_mac(s[3], a, y2x); fx_mac(s[3], d, y1y); fx_mac(s[4], b, y2y); fx_mac(s[4], c, y1x);
+    fx_mac(s[5], a, y2y); fx_mac(s[5], b, y2x); fx_mac(s[6], c, y1y); fx_mac(s[6], d, y1x);
+  };
+  for (int64_t p0 = 0; p0 < h; p0 += 512) {
+    const int pe = (int)min((int64_t)512, h - p0);
+    const int4* y1 = yl + p0;
+    const int4* y2 = yl + h + p0;
+    int4 keep = make_int4(0, 0, 0, 0);
+    int k = 0;
+    for (int i = w; i <= j; i += nw) {
+      const fxc* v = V + (int64_t)i * n + p0;
+      FxAcc s[7];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (cb + q < c1) {
-              const double z = Z[(size_t)(cb + q) * m + i];
-              ar[q] = fma(v.x, z, ar[q]);
-              ai[q] = fma(v.y, z, ai[q]);
-            }
-          }
+      for (int t = 0; t < 7; ++t) fx_zero(s[t]);
+      int p = lane;
+#pragma unroll 1
+      for (; p + 32 < pe; p += 64) {
+        const fxc a1 = v[p], a2 = v[h + p], b1 = v[p + 32], b2 = v[h + p + 32];
+        pair(s, a1, a2, y1[p], y2[p]);
+        pair(s, b1, b2, y1[p + 32], y2[p + 32]);
+      }
+      if (p < pe) pair(s, v[p], v[h + p], y1[p], y2[p]);
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int4 q = fx_warp_sum(t == 0 ? s[0] : fx_diff(s[2 * t - 1], s[2 * t]));
+        if (lane == 4 * k + t) keep = q;
+      }
+      if (++k == 8 || i + nw > j) {
+        const int il = i - nw * (k - 1 - (lane >> 2));       // this lane's column
+        if ((lane >> 2) < k) {
+          const double u = fx_value(keep, vexp[il], Ky);
+          double* out = coef + 4 * il + (lane & 3);
+          *out = p0 == 0 ? u : *out + u;
+        }
+        k = 0;
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// y -= V c_v + W c_w; returns ||y||^2 (block-wide) and the high word of y's largest |component| in *ymax.
+// The columns are split as in gsfx.cu (UpdFx): those with a component above 2^-30 ||y|| / ((j+1)(j+4)) in
+// full, the others by the leading limb of V and 22 bits of the coefficient.  G groups of hp threads share
+// the small columns; group 0 adds their sums (part: 4 integers a thread), takes the large ones and y.
+__device__ double cta_update_fx(const fxc* V, const double* coef, FxState& F, FxCoef u, double* red, int64_t n, int64_t h, int j, double ynorm, double2* y,
+                                long long* part, int gs_groups, int* ymax) {
+  if (threadIdx.x < 32) {                                  // classify and convert the coefficients (j < 64)
+    const int lane = threadIdx.x;
+    const float thr = (float)ynorm * (9.3132257e-10f / ((float)(j + 1) * (float)(j + 4)));
+    int fs = 0, fl = 0, g[3];
+    bool large[3];
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      const int i = lane + 32 * w;
+      g[w] = 0;
+      large[w] = false;
+      if (i <= j) {
+        const double* c = coef + 4 * i;
+        const float mx = fmaxf(fmaxf(fabsf((float)c[0]), fabsf((float)c[1])), fmaxf(fabsf((float)c[2]), fabsf((float)c[3])));
+        const int f = max(max(fx_field(c[0]), fx_field(c[1])), max(fx_field(c[2]), fx_field(c[3])));
+        g[w] = f ? max(f + F.vexp[i] - 1023, 1) : 0;
+        large[w] = !(mx <= thr);
+        if (large[w]) fl = max(fl, g[w]);
+        else fs = max(fs, g[w]);
+      }
+    }
+    const int KS = __reduce_max_sync(0xffffffffu, fs) + 1, KL = __reduce_max_sync(0xffffffffu, fl) + 1;
+    int cnt = 0;
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      const int i = lane + 32 * w;
+      const unsigned b = __ballot_sync(0xffffffffu, large[w]);
+      if (i <= j) {
+        const double* c = coef + 4 * i;
+        const int e = F.vexp[i] - 1023;
+        if (large[w]) {
+          const fx2 p = fx_limbs<true>(c[0], KL - e), q = fx_limbs<true>(c[1], KL - e);
+          const fx2 r = fx_limbs<true>(c[2], KL - e), t = fx_limbs<true>(c[3], KL - e);
+          u.lg[2 * i] = make_int4(p.h, p.l, q.h, q.l);
+          u.lg[2 * i + 1] = make_int4(r.h, r.l, t.h, t.l);
+          u.sm[i] = make_int4(0, 0, 0, 0);
+          u.list[cnt + __popc(b & ((1u << lane) - 1u))] = i;
         } else {
-          const float4 v = ((const float4*)Vv)[(int64_t)i * n + p];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (cb + q < c1) {
-              const float2 z = Zf[(size_t)(cb + q) * m + i];
-              b_df_acc(sr[q], er[q], v.x, v.z, z.x, z.y);
-              b_df_acc(si[q], ei[q], v.y, v.w, z.x, z.y);
-            }
-          }
+          u.sm[i] = make_int4((fx_limbs<true>(c[0], KS - e).h + 32) >> 6, (fx_limbs<true>(c[1], KS - e).h + 32) >> 6,
+                              (fx_limbs<true>(c[2], KS - e).h + 32) >> 6, (fx_limbs<true>(c[3], KS - e).h + 32) >> 6);
         }
       }
+      cnt += __popc(b);
+    }
+    if (lane == 0) {
+      F.misc[0] = cnt;
+      F.misc[1] = KS;
+      F.misc[2] = KL;
+    }
+  }
+  __syncthreads();
+  const int nl = F.misc[0], KS = F.misc[1], KL = F.misc[2];
+  double nrm = 0.0;
+  int ym = 0;
+  auto small_sums = [&](int64_t p, int g0, int G, long long* s) {
+    s[0] = s[1] = s[2] = s[3] = 0;
+    const fxc* v = V + p;
+#pragma unroll 4
+    for (int i = g0; i <= j; i += G) {
+      const fxc v1 = v[(int64_t)i * n], v2 = v[(int64_t)i * n + h];
+      const int4 c = u.sm[i];
+      const int ax = (int)(v1.re >> 32), ay = (int)(v1.im >> 32), bx = (int)(v2.re >> 32), by = (int)(v2.im >> 32);
+      const int ny = -c.y, nz = -c.z, nw = -c.w;
+      fx_mad(s[0], ax, c.x); fx_mad(s[0], ay, ny); fx_mad(s[0], bx, nz); fx_mad(s[0], by, nw);
+      fx_mad(s[1], ax, c.y); fx_mad(s[1], ay, c.x); fx_mad(s[1], bx, nw); fx_mad(s[1], by, c.z);
+      fx_mad(s[2], bx, c.x); fx_mad(s[2], by, ny); fx_mad(s[2], ax, c.z); fx_mad(s[2], ay, c.w);
+      fx_mad(s[3], bx, c.y); fx_mad(s[3], by, c.x); fx_mad(s[3], ax, c.w); fx_mad(s[3], ay, nz);
+    }
+  };
+  auto apply = [&](int64_t p, const long long* s) {
+    double d[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (cb + q < c1) {
-          Vt[(int64_t)(cb + q) * n + p] = DF ? make_double2((double)sr[q] + (double)er[q], (double)si[q] + (double)ei[q])
-                                             : make_double2(ar[q], ai[q]);
-        }
+    for (int t = 0; t < 4; ++t) d[t] = fx_to_double(s[t] >> 63, (unsigned long long)s[t], KS - 1023 - 50);
+    for (int l0 = 0; l0 < nl; l0 += 16) {                  // at most 64 products a sum
+      FxAcc f[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) fx_zero(f[t]);
+      for (int l = l0; l < min(nl, l0 + 16); ++l) {
+        const int k = u.list[l];
+        const fxc v1 = V[(int64_t)k * n + p], v2 = V[(int64_t)k * n + h + p];
+        const int4 cv = u.lg[2 * k], cw = u.lg[2 * k + 1];
+        const fx2 a = fx_round(v1.re), b = fx_round(v1.im), c = fx_round(v2.re), e = fx_round(v2.im);
+        const fx2 P{cv.x, cv.y}, Q{cv.z, cv.w}, R{cw.x, cw.y}, T{cw.z, cw.w};
+        const fx2 nq = fx_neg(Q), nr = fx_neg(R), nt = fx_neg(T);
+        fx_mac(f[0], a, P); fx_mac(f[0], b, nq); fx_mac(f[0], c, nr); fx_mac(f[0], e, nt);
+        fx_mac(f[1], a, Q); fx_mac(f[1], b, P); fx_mac(f[1], c, nt); fx_mac(f[1], e, R);
+        fx_mac(f[2], c, P); fx_mac(f[2], e, nq); fx_mac(f[2], a, R); fx_mac(f[2], b, T);
+        fx_mac(f[3], c, Q); fx_mac(f[3], e, P); fx_mac(f[3], a, T); fx_mac(f[3], b, nr);
       }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) d[t] += fx_lane_value(f[t], KL);
+    }
+    double2 y1 = y[p], y2 = y[h + p];
+    y1.x -= d[0]; y1.y -= d[1];
+    y2.x -= d[2]; y2.y -= d[3];
+    y[p] = y1;
+    y[h + p] = y2;
+    nrm += cabs2(y1) + cabs2(y2);
+    ym = max(ym, max(max(__double2hiint(y1.x) & 0x7fffffff, __double2hiint(y1.y) & 0x7fffffff),
+                     max(__double2hiint(y2.x) & 0x7fffffff, __double2hiint(y2.y) & 0x7fffffff)));
+  };
+  const int hp = (int)(((h + 31) >> 5) << 5);
+  long long s[4];
+  if (hp <= (int)blockDim.x) {
+    int G = (int)blockDim.x / hp;
+    if (gs_groups > 0 && G > gs_groups) G = gs_groups;
+    const int g = (int)threadIdx.x / hp, tl = (int)threadIdx.x - g * hp;
+    const bool active = g < G && tl < h;
+    if (active) small_sums(tl, g, G, s);
+    if (G > 1) {
+      if (active && g > 0)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) part[(size_t)t * blockDim.x + (g - 1) * hp + tl] = s[t];
+      __syncthreads();
+      if (active && g == 0)
+        for (int gg = 1; gg < G; ++gg)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) s[t] += part[(size_t)t * blockDim.x + (gg - 1) * hp + tl];
+    }
+    if (active && g == 0) apply(tl, s);
+  } else {
+    for (int64_t p = threadIdx.x; p < h; p += blockDim.x) {
+      small_sums(p, 0, 1, s);
+      apply(p, s);
+    }
+  }
+  *ymax = blk_imax(ym, F.imax);
+  return blk_isum(nrm, red);
+}
+
+// Z (m x kk) as limbs on one K a column, scaled by the columns' 2^e of V; a unit column is noted.
+__device__ void cta_zlimbs(FxState& S, const double* Z, int m, int kk, int2* zl) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int c = w; c < kk; c += nw) {
+    int f = 0, cnt = 0, unit = m;
+    for (int k = lane; k < m; k += 32) {
+      const double z = Z[(size_t)c * m + k];
+      const int g = fx_field(z);
+      f = max(f, g ? max(g + S.vexp[k] - 1023, 1) : 0);
+      if (g >= 1023 - 60) {
+        ++cnt;
+        unit = __double2hiint(z) < 0 ? ~k : k;
+      }
+    }
+    const int K = __reduce_max_sync(0xffffffffu, f) + 1;
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    const unsigned has = __ballot_sync(0xffffffffu, unit != m);
+    if (has) unit = __shfl_sync(0xffffffffu, unit, __ffs(has) - 1);
+    for (int k = lane; k < m; k += 32) {
+      const fx2 t = fx_limbs<true>(Z[(size_t)c * m + k], K - (S.vexp[k] - 1023));
+      zl[(size_t)c * m + k] = make_int2(t.h, t.l);
+    }
+    if (lane == 0) {
+      S.zk[c] = K;
+      S.zunit[c] = cnt == 1 ? unit : m;
+    }
+  }
+  __syncthreads();
+}
+
+// Vt[:, c] = V Z[:, c], c0 <= c < c1 (m <= 64 products a sum): a thread a row and four columns.
+__device__ void cta_rotate_fx(const fxc* V, const FxState& S, int64_t n, int m, const int2* zl, int c0, int c1, double2* Vt) {
+  const int64_t quads = (c1 - c0 + 3) / 4;
+  for (int64_t q = threadIdx.x; q < n * quads; q += blockDim.x) {
+    const int64_t p = q % n;
+    const int cb = c0 + 4 * (int)(q / n);
+    FxAcc a[4][2];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      fx_zero(a[t][0]);
+      fx_zero(a[t][1]);
+    }
+#pragma unroll 2
+    for (int k = 0; k < m; ++k) {
+      const fxc x = V[(int64_t)k * n + p];
+      const fx2 re = fx_round(x.re), im = fx_round(x.im);
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (cb + t < c1) {
+          const int2 z = zl[(size_t)(cb + t) * m + k];
+          fx_mac(a[t][0], re, fx2{z.x, z.y});
+          fx_mac(a[t][1], im, fx2{z.x, z.y});
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (cb + t < c1) {
+        const int u = S.zunit[cb + t], k = u < 0 ? ~u : u;
+        double2 o;
+        if (k < m) {
+          const fxc x = V[(int64_t)k * n + p];
+          const double re = fx_load(x.re, S.vexp[k]), im = fx_load(x.im, S.vexp[k]);
+          o = u < 0 ? make_double2(-re, -im) : make_double2(re, im);
+        } else {
+          o = make_double2(fx_lane_value(a[t][0], S.zk[cb + t]), fx_lane_value(a[t][1], S.zk[cb + t]));
+        }
+        Vt[(int64_t)(cb + t) * n + p] = o;
+      }
+  }
+  __syncthreads();
+}
+
+// V[:, c] = Vt[:, perm[c]] with its exponent for c < k (a warp a column), V[:, k] = V[:, m].
+__device__ void cta_store_fx(fxc* V, FxState& S, const int* perm, const double2* Vt, int64_t n, int k, int m) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int c = w; c <= k; c += nw) {
+    fxc* dst = V + (int64_t)c * n;
+    if (c < k) {
+      const double2* src = Vt + (int64_t)perm[c] * n;
+      int ex = 0;
+      for (int64_t p = lane; p < n; p += 32) ex = max(ex, max(fx_field(src[p].x), fx_field(src[p].y)));
+      const int K = __reduce_max_sync(0xffffffffu, ex) + 1;
+      for (int64_t p = lane; p < n; p += 32) dst[p] = fxc{fx_store(src[p].x, K), fx_store(src[p].y, K)};
+      if (lane == 0) S.vexp[c] = K;
+    } else {
+      const fxc* src = V + (int64_t)m * n;
+      for (int64_t p = lane; p < n; p += 32) dst[p] = src[p];
+      if (lane == 0) S.vexp[c] = S.vexp[m];
     }
   }
   __syncthreads();
@@ -925,13 +1190,20 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_kernel(BatchArgs a) {
     const int inst = a.order[qi];
     const int64_t h = a.h[inst], n = 2 * h, off = a.a_off[inst];
     auto vcol = [&](int c) -> char* { return (char*)V + (size_t)c * n * 16; };
-    auto store_v = [&](int c, int64_t p, double2 v) {
-      if (DF) ((float4*)vcol(c))[p] = b_split(v);
-      else ((double2*)vcol(c))[p] = v;
-    };
+    auto total = [&](double v) { return DF ? blk_sum(v, S.red) : blk_isum(v, S.red); };
+    const int Ka = DF ? 0 : a.aexp[inst];                 // K of the integer form's A
+    int4* xl = (int4*)x4;                                 // limbs of x, and of y during Gram-Schmidt
+    FxState& F = *(FxState*)S.coef4;
+    const FxCoef fc{(int4*)zb, (int4*)zb + (m + 1), (int*)((int4*)zb + 3 * (m + 1))};
     // ---- v_1 = (1, ..., 1) / sqrt(n) (Algorithm 1); T-bar = 0
     const double v0 = 1.0 / sqrt((double)n);
-    for (int64_t p = threadIdx.x; p < n; p += blockDim.x) store_v(0, p, make_double2(v0, 0.0));
+    if constexpr (DF) {
+      for (int64_t p = threadIdx.x; p < n; p += blockDim.x) ((float4*)V)[p] = b_split(make_double2(v0, 0.0));
+    } else {
+      const int K = fx_field(v0) + 1;
+      for (int64_t p = threadIdx.x; p < n; p += blockDim.x) ((fxc*)V)[p] = fxc{fx_store(v0, K), 0};
+      if (threadIdx.x == 0) F.vexp[0] = K;
+    }
     for (int e = threadIdx.x; e < ldt * ldt; e += blockDim.x) T[e] = 0.0;
     if (threadIdx.x == 0) {
       S.k = 0; S.icnv = 0; S.status = 0; S.tmax = 0.0; S.nlocked = 0;
@@ -953,20 +1225,24 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_kernel(BatchArgs a) {
       // ---- Algorithm 2: Lanczos steps k .. m-1
       for (int j = k; j < m; ++j) {
         for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
-          if (DF) {
+          if constexpr (DF) {
             const float4 v = ((const float4*)vcol(j))[p];
             x4[p] = v;
             x[p] = b_join(v);
           } else {
-            x[p] = ((const double2*)vcol(j))[p];
+            const fxc v = ((const fxc*)vcol(j))[p];
+            const fx2 re = fx_round(v.re), im = fx_round(v.im);
+            xl[p] = make_int4(re.h, re.l, im.h, im.l);
+            x[p] = make_double2(fx_load(v.re, F.vexp[j]), fx_load(v.im, F.vexp[j]));
           }
         }
         __syncthreads();
-        cta_matvec<DF, MVR>(a, h, off, x, x4, y, S.red);
+        if constexpr (DF) cta_matvec<MVR>(a, h, off, x4, y);
+        else cta_matvec_fx((const fxc*)a.A11 + off, (const fxc*)a.A12 + off, h, xl, F.vexp[j], Ka, y);
         ++n_mv;
         double al = 0.0;
         for (int64_t p = threadIdx.x; p < n; p += blockDim.x) al += x[p].x * y[p].x + x[p].y * y[p].y;
-        al = blk_sum(al, S.red);                                  // t_{j,j} = Re(v_j^H A v_j)
+        al = total(al);                                           // t_{j,j} = Re(v_j^H A v_j)
         double nrm = 0.0;
         for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
           double2 t = y[p];
@@ -975,11 +1251,18 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_kernel(BatchArgs a) {
           y[p] = t;
           nrm += cabs2(t);
         }
-        double b0 = sqrt(blk_sum(nrm, S.red)), b1 = b0;
+        double b0 = sqrt(total(nrm)), b1 = b0;
+        int ymax = 0;
         mark(0);
         for (int pass = 0; pass < a.gs_passes; ++pass) {         // against W_j and V_j, sqrt(2) test
-          cta_dot<DF>(V, n, h, j, y, x4, S.coef, S.coef4);
-          b1 = sqrt(cta_update<DF>(V, n, h, j, S.coef, S.coef4, y, part, S.red, a.gs_groups));
+          if constexpr (DF) {
+            cta_dot((const float4*)V, n, h, j, y, x4, S.coef, S.coef4);
+            b1 = sqrt(cta_update((const float4*)V, n, h, j, S.coef4, y, part, S.red, a.gs_groups));
+          } else {
+            const int Ky = cta_limbs(y, n, xl, F.imax);
+            cta_dot_fx((const fxc*)V, F.vexp, n, h, j, xl, Ky, S.coef);
+            b1 = sqrt(cta_update_fx((const fxc*)V, S.coef, F, fc, S.red, n, h, j, b0, y, (long long*)part, a.gs_groups, &ymax));
+          }
           ++n_gs;
           if (sqrt2 * b1 > b0) break;
           b0 = b1;
@@ -987,7 +1270,15 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_kernel(BatchArgs a) {
         const double tmax = fmax(S.tmax, fmax(fabs(al), b1));
         const bool brk = !(b1 > 1e-14 * fmax(tmax, 1.0));
         const double inv = brk ? 0.0 : 1.0 / b1;
-        for (int64_t p = threadIdx.x; p < n; p += blockDim.x) store_v(j + 1, p, make_double2(y[p].x * inv, y[p].y * inv));
+        if constexpr (DF) {
+          for (int64_t p = threadIdx.x; p < n; p += blockDim.x)
+            ((float4*)vcol(j + 1))[p] = b_split(make_double2(y[p].x * inv, y[p].y * inv));
+        } else {
+          const int K = fx_field(__hiloint2double(ymax + 1, 0) * inv) + 1;
+          for (int64_t p = threadIdx.x; p < n; p += blockDim.x)
+            ((fxc*)vcol(j + 1))[p] = fxc{fx_store(y[p].x * inv, K), fx_store(y[p].y * inv, K)};
+          if (threadIdx.x == 0) F.vexp[j + 1] = K;
+        }
         __syncthreads();
         if (threadIdx.x == 0) {
           T[j * ldt + j] = al;
@@ -1021,14 +1312,17 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_kernel(BatchArgs a) {
       }
       mark(2);
       // ---- V_m Z for the nev candidates; Krylov-Schur arrow t_{m+1,i} = beta_m z_{m,i}
-      if (DF) {
+      if constexpr (DF) {
         for (int e = threadIdx.x; e < kk * m; e += blockDim.x) {
           const float zh = (float)Z[e];
           Zf[e] = make_float2(zh, (float)(Z[e] - (double)zh));
         }
         __syncthreads();
+        cta_rotate((const float4*)V, n, m, Zf, 0, nev, Vt);
+      } else {
+        cta_zlimbs(F, Z, m, kk, (int2*)Zf);
+        cta_rotate_fx((const fxc*)V, F, n, m, (const int2*)Zf, 0, nev, Vt);
       }
-      cta_rotate<DF>(V, n, m, Z, Zf, 0, nev, Vt);
       if (threadIdx.x == 0) {
         for (int i = 0; i < kk; ++i) {
           S.lamv[i] = S.lam[i];
@@ -1067,14 +1361,19 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_kernel(BatchArgs a) {
           if (DF) x4[p] = b_split(v);
         }
         __syncthreads();
-        cta_matvec<DF, MVR>(a, h, off, x, x4, y, S.red);
+        if constexpr (DF) {
+          cta_matvec<MVR>(a, h, off, x4, y);
+        } else {
+          const int Kx = cta_limbs(x, n, xl, F.imax);
+          cta_matvec_fx((const fxc*)a.A11 + off, (const fxc*)a.A12 + off, h, xl, Kx, Ka, y);
+        }
         ++n_res;
         double rr = 0.0;
         for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
           const double dr = y[p].x - S.ev[i] * x[p].x, di = y[p].y - S.ev[i] * x[p].y;
           rr += dr * dr + di * di;
         }
-        rr = sqrt(blk_sum(rr, S.red));
+        rr = sqrt(total(rr));
         if (threadIdx.x == 0) {
           S.res[i] = rr;
           S.conv[i] = rr < a.tol;
@@ -1124,12 +1423,15 @@ __global__ void __launch_bounds__(kBatchMaxThreads) batch_kernel(BatchArgs a) {
       }
       // ---- shrink: kept columns (rotated, permuted) into V, v_{k+1} = v_{m+1}, arrowhead T-bar
       const int knew = S.k;
-      cta_rotate<DF>(V, n, m, Z, Zf, nev, knew, Vt);
-      for (int c = 0; c < knew; ++c)
-        for (int64_t p = threadIdx.x; p < n; p += blockDim.x) store_v(c, p, Vt[(int64_t)S.perm[c] * n + p]);
-      for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
-        if (DF) ((float4*)vcol(knew))[p] = ((const float4*)vcol(m))[p];
-        else ((double2*)vcol(knew))[p] = ((const double2*)vcol(m))[p];
+      if constexpr (DF) {
+        cta_rotate((const float4*)V, n, m, Zf, nev, knew, Vt);
+        for (int c = 0; c < knew; ++c)
+          for (int64_t p = threadIdx.x; p < n; p += blockDim.x)
+            ((float4*)vcol(c))[p] = b_split(Vt[(int64_t)S.perm[c] * n + p]);
+        for (int64_t p = threadIdx.x; p < n; p += blockDim.x) ((float4*)vcol(knew))[p] = ((const float4*)vcol(m))[p];
+      } else {
+        cta_rotate_fx((const fxc*)V, F, n, m, (const int2*)Zf, nev, knew, Vt);
+        cta_store_fx((fxc*)V, F, S.perm, Vt, n, knew, m);
       }
       for (int e = threadIdx.x; e < ldt * ldt; e += blockDim.x) T[e] = 0.0;
       __syncthreads();
@@ -1193,6 +1495,29 @@ __global__ void split_df_inplace_kernel(double2* A, int64_t count) {
   }
 }
 
+// K of each instance's blocks (both on one): 1 + the largest exponent field, into the zeroed aexp.
+__global__ void batch_field_kernel(const double2* A11, const double2* A12, const int64_t* h, const int64_t* off, int* aexp) {
+  const int inst = blockIdx.y;
+  const int64_t cnt = h[inst] * h[inst], o = off[inst];
+  int ex = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
+    const double2 a = A11[o + i], b = A12[o + i];
+    ex = max(ex, max(max(fx_field(a.x), fx_field(a.y)), max(fx_field(b.x), fx_field(b.y))));
+  }
+  ex = __reduce_max_sync(0xffffffffu, ex);
+  if ((threadIdx.x & 31) == 0) atomicMax(aexp + inst, ex + 1);
+}
+// FP64 blocks to fixed point, in place.
+__global__ void batch_fix_kernel(double2* A11, double2* A12, const int64_t* h, const int64_t* off, const int* aexp) {
+  const int inst = blockIdx.y, K = aexp[inst];
+  const int64_t cnt = h[inst] * h[inst], o = off[inst];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
+    const double2 a = A11[o + i], b = A12[o + i];
+    ((fxc*)A11)[o + i] = fxc{fx_store(a.x, K), fx_store(a.y, K)};
+    ((fxc*)A12)[o + i] = fxc{fx_store(b.x, K), fx_store(b.y, K)};
+  }
+}
+
 __global__ void c64_to_c128_batch_kernel(const float2* in, double2* out, int64_t count) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = make_double2((double)in[i].x, (double)in[i].y);
@@ -1205,7 +1530,7 @@ size_t batch_smem_bytes(int64_t nmax, int m, int kk, int threads) { return Batch
 namespace {
 const void* batch_fn(bool df, int mv_rows) {
   if (df) return mv_rows == 1 ? (const void*)batch_kernel<true, 1> : (const void*)batch_kernel<true, 2>;
-  return mv_rows == 2 ? (const void*)batch_kernel<false, 2> : (const void*)batch_kernel<false, 1>;
+  return (const void*)batch_kernel<false, 1>;   // a warp takes one row at a time
 }
 }  // namespace
 
@@ -1222,8 +1547,7 @@ cudaError_t launch_batch(bool df, const BatchArgs& a, int grid, int threads, cud
     if (a.mv_rows == 1) batch_kernel<true, 1><<<grid, threads, sm, s>>>(a);
     else batch_kernel<true, 2><<<grid, threads, sm, s>>>(a);
   } else {
-    if (a.mv_rows == 2) batch_kernel<false, 2><<<grid, threads, sm, s>>>(a);
-    else batch_kernel<false, 1><<<grid, threads, sm, s>>>(a);
+    batch_kernel<false, 1><<<grid, threads, sm, s>>>(a);
   }
   return cudaGetLastError();
 }
@@ -1231,6 +1555,18 @@ cudaError_t launch_batch(bool df, const BatchArgs& a, int grid, int threads, cud
 cudaError_t launch_split_df_inplace(void* A, int64_t count, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   split_df_inplace_kernel<<<1024, 256, 0, s>>>((double2*)A, count);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_fix(void* A11, void* A12, const int64_t* h, const int64_t* off, int count, int* aexp,
+                             cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(aexp, 0, (size_t)count * sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  for (int i = 0; i < count; i += 32768) {             // the grid's second extent is below 65536
+    const dim3 grid(16, count - i < 32768 ? count - i : 32768);
+    batch_field_kernel<<<grid, 256, 0, s>>>((const double2*)A11, (const double2*)A12, h + i, off + i, aexp + i);
+    batch_fix_kernel<<<grid, 256, 0, s>>>((double2*)A11, (double2*)A12, h + i, off + i, aexp + i);
+  }
   return cudaGetLastError();
 }
 

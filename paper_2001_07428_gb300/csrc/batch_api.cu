@@ -59,6 +59,7 @@ struct jtrlan_batch {
   long long* prof = nullptr;    // per-instance phase cycles (params.profile)
   void* out_vec = nullptr;
   int* queue = nullptr;
+  int* aexp = nullptr;
   int n_sm = 0;
   int threads = 256;
   int ctas_per_sm = 0;          // 0: as many as fit
@@ -193,6 +194,8 @@ jtrlan_status create_batch(int count, const jtrlan_operator* ops, const jtrlan_p
   JB_TRY(b->dalloc(&b->out_vec, (size_t)v_total * sizeof(double2)));
   JB_TRY(b->dalloc(&vp, sizeof(int)));
   b->queue = (int*)vp;
+  JB_TRY(b->dalloc(&vp, (size_t)count * sizeof(int)));
+  b->aexp = (int*)vp;
   JB_CUDA(cudaMemcpyAsync(b->d_order, b->order.data(), count * sizeof(int), cudaMemcpyHostToDevice, b->own));
   JB_CUDA(cudaMemcpyAsync(b->d_h, b->h.data(), count * sizeof(int64_t), cudaMemcpyHostToDevice, b->own));
   JB_CUDA(cudaMemcpyAsync(b->d_aoff, b->a_off.data(), count * sizeof(int64_t), cudaMemcpyHostToDevice, b->own));
@@ -210,6 +213,8 @@ jtrlan_status create_batch(int count, const jtrlan_operator* ops, const jtrlan_p
   if (b->df) {
     JB_CUDA(launch_split_df_inplace(b->A11, a_total, b->own));
     JB_CUDA(launch_split_df_inplace(b->A12, a_total, b->own));
+  } else {
+    JB_CUDA(launch_batch_fix(b->A11, b->A12, b->d_h, b->d_aoff, count, b->aexp, b->own));
   }
   JB_CUDA(cudaStreamSynchronize(b->own));  // the caller may free its blocks after this call
   b->release(tmp);
@@ -251,6 +256,7 @@ BatchArgs args_of(const jtrlan_batch* b) {
   a.a_off = b->d_aoff;
   a.A11 = b->A11;
   a.A12 = b->A12;
+  a.aexp = b->aexp;
   a.Vslots = b->slots_v;
   a.Tslots = b->slots_t;
   a.nmax = b->nmax;

@@ -177,6 +177,20 @@ __device__ __forceinline__ double fx_warp_dsum(const double* src, int stride, in
   return fx_to_double(hi, lo, K - 1023 - 56 + 2);
 }
 
+// Sum of one double a lane, as fx_warp_dsum; every lane gets it.
+__device__ __forceinline__ double fx_warp_total(double v) {
+  const int ex = __reduce_max_sync(0xffffffffu, fx_field(v));
+  if (ex == 0x7ff) return warp_sum(v);
+  const int K = ex + 1;
+  const fx2 t = fx_limbs<true>(v, K);
+  const unsigned w = __reduce_add_sync(0xffffffffu, (unsigned)t.l >> 2);          // units 2^2
+  const int a = __reduce_add_sync(0xffffffffu, t.h >> 14), b = __reduce_add_sync(0xffffffffu, t.h & 0x3fff);
+  const long long hs = ((long long)a << 14) + b;                                  // units 2^28
+  const unsigned long long lo = ((unsigned long long)hs << 26) + w;
+  const long long hi = (hs >> 38) + (lo < (unsigned long long)w ? 1 : 0);
+  return fx_to_double(hi, lo, K - 1023 - 56 + 2);
+}
+
 __device__ __forceinline__ double fx_load(long long F, int K) { return fx_to_double(F >> 63, (unsigned long long)F, K - 1023 - 60); }
 
 }  // namespace jtr

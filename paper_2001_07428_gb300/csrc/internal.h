@@ -225,6 +225,7 @@ struct BatchArgs {
   const int64_t* a_off;
   const void* A11;
   const void* A12;
+  const int* aexp;   // FP64 form: K of each instance's fixed-point blocks
   void* Vslots;
   void* Tslots;
   int64_t nmax;
@@ -251,6 +252,9 @@ cudaError_t launch_batch(bool df, const BatchArgs& a, int grid, int threads, cud
 // In place: each double2 element becomes the float4 (hi.re, hi.im, lo.re, lo.im) with hi = fl32(x),
 // lo = fl32(x - hi).
 cudaError_t launch_split_df_inplace(void* A, int64_t count, cudaStream_t s);
+// In place: the FP64 blocks become fixed point (fxc of fixed.cuh), one K per instance into aexp.
+cudaError_t launch_batch_fix(void* A11, void* A12, const int64_t* h, const int64_t* off, int count, int* aexp,
+                             cudaStream_t s);
 cudaError_t launch_c64_to_c128(const void* in, void* out, int64_t count, cudaStream_t s);
 
 // ------------------------------------------------------------------ polynomial filter (filter.cu)
