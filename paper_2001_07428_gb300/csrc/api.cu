@@ -93,6 +93,8 @@ struct Profiler {
 // Operator copy and Krylov basis in one working precision.
 struct Phase {
   OpDev op{};
+  OpDev opfx{};           // plain FP64, stencil: fixed-point links for the Lanczos products
+  bool fxmv = false;      // use opfx
   OpDev opdf{};           // double-float phase, stencil: (hi, lo) links for the Lanczos products
   bool dfmv = false;      // use opdf for the Lanczos products
   void* V = nullptr;      // n x (m + 1): FP32, (hi, lo) float4 pairs (df), or the fixed-point basis (fx)
@@ -351,6 +353,29 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
     c->p64.fx = true;
     JT_TRY(make_phase(c->p64, sizeof(double2)));
     JT_TRY(c->dalloc(&c->p64.x, (size_t)c->n * sizeof(double2)));
+    if (op->kind == JTRLAN_STENCIL4D && c->n < (int64_t)1 << 31) {   // fixed-point links; 32-bit sites and entries
+      OpDev& d = c->p64.opfx;
+      d = o;
+      int* kfx = nullptr;
+      void* uw = nullptr;
+      const size_t bytes = (size_t)36 * o.vol * 16;
+      if (cudaMalloc(&uw, 2 * bytes) == cudaSuccess) {   // without room for them the FP64 kernel serves
+        c->owned.push_back(uw);
+        JT_TRY(c->dalloc(&kfx, 2 * sizeof(int)));
+        d.U = uw;
+        d.W = (char*)uw + bytes;
+        d.kfx = kfx;
+        JT_CUDA(launch_field(o.U, 36 * o.vol, kfx, c->stream));
+        JT_CUDA(launch_field(o.W, 36 * o.vol, kfx + 1, c->stream));
+        JT_CUDA(launch_links_fx(o.U, (void*)d.U, o.vol, kfx, c->stream));
+        JT_CUDA(launch_links_fx(o.W, (void*)d.W, o.vol, kfx + 1, c->stream));
+        c->p64.fxmv = true;
+      } else {
+        cudaGetLastError();
+      }
+      if (c->p64.fxmv && matvec_fx_blocks(d) > c->p64.mv_nblk)
+        JT_TRY(c->dalloc(&c->p64.alpha_part, (size_t)matvec_fx_blocks(d) * sizeof(double2)));
+    }
   } else {  // double-float phase on the FP64 operator
     c->pdf.op = o;
     c->pdf.df = true;
@@ -731,7 +756,8 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
   if (ph.fx) LAUNCH(K_OTHER, launch_load_col(ph.V, c->vexp, n, j0, (double2*)ph.x, s));
   const int mv_parts = c->invert ? cg_blocks(n)
                        : (filtered && !(ph.certify && ph.dfmv)) ? cheb_blocks(n)
-                       : ph.dfmv ? matvec_df_blocks(ph.opdf) : ph.mv_nblk;
+                       : ph.dfmv ? matvec_df_blocks(ph.opdf)
+                       : ph.fxmv && !filtered ? matvec_fx_blocks(ph.opfx) : ph.mv_nblk;
   for (int j = j0; j < j1; ++j) {
     if (filtered) {
       if constexpr (std::is_same<R, float>::value)
@@ -743,6 +769,8 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
     } else if (c->invert) {   // invert mode: y = A^{-1} v_j by CG, then the partials of v_j^H y
       JT_TRY(cg_solve(c, ph, ph.x, ph.y));
       LAUNCH(K_CG, launch_vhy_part(ph.x, ph.y, n, ph.alpha_part, s));
+    } else if (ph.fxmv) {
+      LAUNCH(K_MATVEC, launch_matvec_fx(ph.opfx, col(ph.V, n, j, cs), c->vexp + j, ph.x, ph.y, ph.alpha_part, s));
     } else {
       const void* vj = ph.x ? ph.x : col(ph.V, n, j, cs);
       LAUNCH(K_MATVEC, launch_matvec<R>(ph.op, (const C*)vj, (C*)ph.y, MV_ALPHA, ph.alpha_part,

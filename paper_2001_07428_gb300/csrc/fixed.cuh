@@ -93,6 +93,8 @@ __device__ __forceinline__ void fx_mac(FxAcc& a, fx2 x, fx2 y) {
   fx_mad(a.M, x.l, y.h);
   fx_mad(a.L, x.l, y.l);
 }
+__device__ __forceinline__ FxAcc fx_sum(const FxAcc& a, const FxAcc& b) { return FxAcc{a.H + b.H, a.M + b.M, a.L + b.L}; }
+__device__ __forceinline__ FxAcc fx_scale(const FxAcc& a, int sign) { return sign > 0 ? a : FxAcc{-a.H, -a.M, -a.L}; }
 __device__ __forceinline__ FxAcc fx_diff(const FxAcc& a, const FxAcc& b) { return FxAcc{a.H - b.H, a.M - b.M, a.L - b.L}; }
 __device__ __forceinline__ fx2 fx_neg(fx2 a) { return fx2{-a.h, -a.l}; }
 

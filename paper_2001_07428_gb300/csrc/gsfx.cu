@@ -729,6 +729,13 @@ cudaError_t launch_store_cols(void* V, const void* X, int64_t n, const int* perm
   return cudaGetLastError();
 }
 
+cudaError_t launch_field(const void* X, int64_t n, int* kmax, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(kmax, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  col_field_kernel<<<dim3(col_grid(n)), 256, 0, s>>>((const double2*)X, n, nullptr, kmax);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_load_col(const void* V, const int* vexp, int64_t n, int c, double2* x, cudaStream_t s) {
   load_col_kernel<<<col_grid(n) * 4, 256, 0, s>>>((const fxc*)V + (int64_t)c * n, vexp + c, n, x);
   return cudaGetLastError();

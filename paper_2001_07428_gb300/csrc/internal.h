@@ -27,6 +27,7 @@ struct OpDev {
   const void* U;       // stencil links: FP64 [4][V][9]; FP32 structure-of-arrays [4][9][V]
   const void* W;
   int fp32;            // 1: FP32 operator (float2 links / blocks), 0: FP64
+  const int* kfx;      // fixed-point links (structure-of-arrays [4][9][V] of fxc): K of U and of W
   int links32;         // compensated-FP32 stencil: 1 = links exact in FP32 (float2 SoA, the caller's
                        // complex64 links), 0 = (hi, lo) float4 SoA
 };
@@ -43,7 +44,14 @@ cudaError_t launch_matvec(const OpDev& op, const cplx<R>* x, cplx<R>* y, MvMode 
                           const int* cand, const double* lam, int ncand, int64_t ldx,
                           int* nblk_out, cudaStream_t s);
 int matvec_blocks(const OpDev& op);  // nblk of launch_matvec for one column
-
+// FP64 stencil product by integer sums (matvec.cu): y = A x for x as fixed point (X on *Kx) and in FP64
+// (x64), fixed-point links in op; part: matvec_fx_blocks double2 partials of x^H y.
+int matvec_fx_blocks(const OpDev& op);
+cudaError_t launch_matvec_fx(const OpDev& op, const void* X, const int* Kx, const void* x64, void* Y, double* part,
+                             cudaStream_t s);
+cudaError_t launch_links_fx(const void* in, void* out, int64_t vol, const int* kfx, cudaStream_t s);
+// *kmax = largest exponent field of the n FP64 complex numbers X + 1
+cudaError_t launch_field(const void* X, int64_t n, int* kmax, cudaStream_t s);
 // Lanczos-step Gram-Schmidt against [V, W] with W = J V^* implicit (Algorithm 2).
 struct GSArgs {
   const void* V;       // n x (m+1) complex, ld = n, working precision

@@ -14,6 +14,7 @@
 // FP64 on this GPU is arithmetic-bound (about 2 DFMA per clock per SM), so the FP64 kernel
 // spreads one site over 24 threads -- (half, colour, direction) -- to keep every SM busy at
 // small volumes; the four direction threads are adjacent lanes and meet through shuffles.
+#include "fixed.cuh"
 #include "internal.h"
 #include "../../include/jtrlan.h"
 
@@ -114,6 +115,115 @@ stencil_kernel(OpDev op, const cplx<R>* __restrict__ X, cplx<R>* __restrict__ Y,
   } else if (MODE == MV_RESID) {
     c0 = block_sum(c0, sh);
     if (threadIdx.x == 0) part[(int64_t)col * gridDim.x + blockIdx.x] = c0;
+  }
+}
+
+// ------------------------------------------------------------------ FP64 by integer sums
+// The FP64 kernel above is bound by the FP64 pipe (79% busy at 8^4).  Here x, U and W are fixed point
+// (fixed.cuh; K of x, one K each for U and W) and the hopping sums exact integer sums, 4 times the FP64
+// rate.  A block is 32 sites by 12 warps, one for each colour a of y1 or y2 and each of its two parts
+// (U terms, W terms), so that a small lattice still fills the SMs; links are structure-of-arrays
+// [4][9][V], so a warp's link load is one 512-byte segment, and the warps share lines of x through L1.
+// Each warp keeps the four real products of forward and of backward hops in sums of their own (12
+// products each) and sets the signs at the end, where the parts meet in FP64:
+//   forward:  y1 U: l x   W: l x         y2 U: l* x   W: -l* x
+//   backward: y1 U: l* x  W: -l x        y2 U: l x    W: l* x
+// 16^4: 207 -> 100 us (waiting for its loads: L1 40% busy, 1.8 instructions a clock), 8^4: 21.0 -> 12.5 us.
+// Per SM: two blocks of 80 registers (a few spill), or one without spills where the lattice has no more
+// blocks than the GPU SMs (8^4: 12.5 against 14.6 us; 16^4: 125 against 100).
+constexpr int kFxSites = 32, kFxWarps = 12;
+
+template <int MinBlocks>
+__global__ void __launch_bounds__(32 * kFxWarps, MinBlocks)
+stencil_fx_kernel(OpDev op, const fxc* __restrict__ X, const int* __restrict__ Kx, const double2* __restrict__ x64,
+                  double2* __restrict__ Y, double* __restrict__ part) {
+  __shared__ double sh[32];
+  __shared__ double2 wsum[6][kFxSites];
+  const int vol = (int)op.vol;
+  const int64_t h = op.h;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int kind = w / 6, half = (w / 3) & 1, a = w % 3;      // kind 0: U, 1: W
+  const int site = blockIdx.x * kFxSites + lane;
+  const int s = min(site, vol - 1);                           // a lane beyond the lattice repeats its last site
+  const fxc* L = (const fxc*)(kind ? op.W : op.U);
+  const fxc* x = X + (half ^ kind ? h : 0);
+  const int kl = op.kfx[kind];
+  FxAcc f[4], b[4];                                           // lr p, li q, lr q, li p
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    fx_zero(f[t]);
+    fx_zero(b[t]);
+  }
+  const int d0 = op.dims[0], d1 = op.dims[1], d2 = op.dims[2], d3 = op.dims[3];
+  const int r1 = s / d0, r2 = r1 / d1;
+  const int c0 = s - r1 * d0, c1 = r1 - r2 * d1, c2 = r2 % d2, c3 = r2 / d2;
+  int stride = 1;
+#pragma unroll 1
+  for (int mu = 0; mu < 4; ++mu) {
+    const int ext = mu == 0 ? d0 : mu == 1 ? d1 : mu == 2 ? d2 : d3;
+    const int c = mu == 0 ? c0 : mu == 1 ? c1 : mu == 2 ? c2 : c3;
+    const int sp = (c == ext - 1) ? s - (ext - 1) * stride : s + stride;
+    const int sm = (c == 0) ? s + (ext - 1) * stride : s - stride;
+    stride *= ext;
+    const fxc* Lm = L + (int64_t)mu * 9 * vol;
+    auto mac = [](FxAcc* g, fxc l, fxc v) {
+      const fx2 lr = fx_round(l.re), li = fx_round(l.im), p = fx_round(v.re), q = fx_round(v.im);
+      fx_mac(g[0], lr, p);
+      fx_mac(g[1], li, q);
+      fx_mac(g[2], lr, q);
+      fx_mac(g[3], li, p);
+    };
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      mac(f, Lm[(int64_t)(a * 3 + e) * vol + s], x[3 * (int64_t)sp + e]);
+      mac(b, Lm[(int64_t)(e * 3 + a) * vol + sm], x[3 * (int64_t)sm + e]);
+    }
+  }
+  // re = sf (f0 - cf f1) + sb (b0 - cb b1), im = sf (f2 + cf f3) + sb (b2 + cb b3); c = -1 conjugates the link
+  const int cf = half ? -1 : 1, cb = kind ? cf : -cf;
+  const int sf = kind && half ? -1 : 1, sb = kind && !half ? -1 : 1;
+  auto comb = [](const FxAcc& p, const FxAcc& q, int sign) { return sign > 0 ? fx_sum(p, q) : fx_diff(p, q); };
+  const FxAcc re = comb(fx_scale(comb(f[0], f[1], -cf), sf), comb(b[0], b[1], -cb), sb);
+  const FxAcc im = comb(fx_scale(comb(f[2], f[3], cf), sf), comb(b[2], b[3], cb), sb);
+  const int kx = *Kx;
+  double2 v = make_double2(fx_lane_value(re, kx + kl - 1023), fx_lane_value(im, kx + kl - 1023));
+  if (kl >= 2048 || kx >= 2048) v = make_double2(NAN, NAN);   // an infinite or NaN link or entry
+  if (kind) wsum[w - 6][lane] = v;
+  __syncthreads();
+  double al = 0.0, ai = 0.0;
+  if (!kind && site < vol) {
+    const double2 u = wsum[w][lane];
+    const int64_t e = (half ? h : 0) + 3 * (int64_t)s + a;
+    const double2 xe = x64[e];
+    v.x += op.kappa * u.x + op.m0 * xe.x;
+    v.y += op.kappa * u.y + op.m0 * xe.y;
+    Y[e] = v;
+    al = xe.x * v.x + xe.y * v.y;   // conj(x_e) y_e
+    ai = xe.x * v.y - xe.y * v.x;
+  }
+  if (!kind) {
+    al = fx_warp_total(al);
+    ai = fx_warp_total(ai);
+    if (lane == 0) {
+      sh[w] = al;
+      sh[6 + w] = ai;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    const double* t = sh + 6 * threadIdx.x;
+    part[2 * blockIdx.x + threadIdx.x] = ((t[0] + t[1]) + (t[2] + t[3])) + (t[4] + t[5]);
+  }
+}
+
+// FP64 links [4][V][9] to fixed point [4][9][V] on K = *kfx.
+__global__ void links_fx_kernel(const double2* in, fxc* out, int64_t vol, const int* kfx) {
+  const int K = *kfx;
+  const int64_t total = 36 * vol;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t s = q % vol, me = q / vol, mu = me / 9, e = me % 9;
+    const double2 v = in[(mu * vol + s) * 9 + e];
+    out[q] = fxc{fx_store(v.x, K), fx_store(v.y, K)};
   }
 }
 
@@ -293,6 +403,25 @@ cudaError_t launch_mode(const OpDev& op, const cplx<R>* x, cplx<R>* y, double* p
 }
 
 }  // namespace
+
+int matvec_fx_blocks(const OpDev& op) { return (int)((op.vol + kFxSites - 1) / kFxSites); }
+
+cudaError_t launch_matvec_fx(const OpDev& op, const void* X, const int* Kx, const void* x64, void* Y, double* part,
+                             cudaStream_t s) {
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int nb = matvec_fx_blocks(op);
+  (nb <= nsm ? stencil_fx_kernel<1> : stencil_fx_kernel<2>)<<<nb, 32 * kFxWarps, 0, s>>>(
+      op, (const fxc*)X, Kx, (const double2*)x64, (double2*)Y, part);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_links_fx(const void* in, void* out, int64_t vol, const int* kfx, cudaStream_t s) {
+  links_fx_kernel<<<1024, 256, 0, s>>>((const double2*)in, (fxc*)out, vol, kfx);
+  return cudaGetLastError();
+}
 
 int matvec_blocks(const OpDev& op) {
   if (op.kind == JTRLAN_STENCIL4D) {
