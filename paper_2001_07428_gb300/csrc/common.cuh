@@ -38,6 +38,34 @@ template <typename C> __device__ __forceinline__ double cabs2(C a) {
 // |a|^2 in the working precision (FP32 partial sums stay on the FP32 pipe)
 template <typename C> __device__ __forceinline__ auto cabs2w(C a) -> decltype(a.x) { return a.x * a.x + a.y * a.y; }
 
+// ------------------------------------------------------------------ dependent launches
+// A step of the method is two or three short kernels, each needing all of the one before, and between two
+// launches of a stream the GPU idles for about 2 us.  A kernel launched by launch_dep may be set up while
+// its predecessor still runs (programmatic dependent launch): it calls dep_wait() before its first access
+// to memory, which returns when every kernel before it has completed and its writes are visible.
+// dep_trigger() in a kernel lets such a successor be set up from there on; it is called after dep_wait(),
+// so at most two kernels of a stream are ever resident.  Data that an earlier kernel wrote is not read
+// through the non-coherent path (no const __restrict__ parameters in these kernels).  A kernel started
+// without the attribute passes both at once.
+// A fused filter step at 9 x 11 x 13 x 15: 14.6 -> 12.2 us, at 16^4 29.0 -> 26.2; a dense solve of order 200,
+// 5.56 -> 5.26 ms.  A cooperative launch does not take the attribute; it only triggers.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ------------------------------------------------------------------ reductions
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

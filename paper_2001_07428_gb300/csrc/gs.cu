@@ -450,6 +450,7 @@ gs_step_coop_kernel(GSArgs a, const double2* __restrict__ alpha_part, int n_alph
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   R* dred = (R*)dyn_smem;
   coef4* sc = (coef4*)(dyn_smem + dot_smem<R>());
+  dep_trigger();   // the next product may be set up from here on
   const int j = a.j;
   const int64_t h = a.h;
   const int nblk = a.nblk;

@@ -530,6 +530,7 @@ gsdf_step_coop_kernel(GSArgs a, double2* __restrict__ x, const double2* __restri
   float* red = (float*)(ys + 2 * a.rows_per_block);
   float4* scf = (float4*)(red + kGroups * 2 * (4 * kCols) * 33);
   const UpdCoef upd{scf, scf + 2 * (a.m + 1), (unsigned char*)(scf + 3 * (a.m + 1))};
+  dep_trigger();   // the next product may be set up from here on
   const int j = a.j;
   const int64_t h = a.h;
   const int nblk = a.nblk;
@@ -882,7 +883,7 @@ struct DfSums {
 
 // The sums in the Dot2 form (the certifying product: residuals and Rayleigh quotients).
 template <typename LinkT>
-__device__ __forceinline__ void stencil_df_sums_dot2(const OpDev& op, const float4* __restrict__ x, int s, int a,
+__device__ __forceinline__ void stencil_df_sums_dot2(const OpDev& op, const float4* x, int s, int a,
                                                 DfSums& r) {
   const int vol = (int)op.vol;
   const int64_t h = op.h;
@@ -934,7 +935,7 @@ __device__ __forceinline__ void stencil_df_sums_dot2(const OpDev& op, const floa
 
 // The sums as biased blocks, one per direction (the Chebyshev steps of the filter).
 template <typename LinkT>
-__device__ __forceinline__ void stencil_df_sums_biased(const OpDev& op, const float4* __restrict__ x, int s, int a,
+__device__ __forceinline__ void stencil_df_sums_biased(const OpDev& op, const float4* x, int s, int a,
                                                 DfSums& r) {
   const int vol = (int)op.vol;
   const int64_t h = op.h;
@@ -1027,8 +1028,10 @@ __device__ __forceinline__ void stencil_df_sums_biased(const OpDev& op, const fl
 
 template <typename LinkT>
 __global__ void __launch_bounds__(3 * kDfSites, kDfMinBlocks)
-stencil_df_kernel(OpDev op, const float4* __restrict__ x, double2* __restrict__ Y, double* __restrict__ part) {
+stencil_df_kernel(OpDev op, const float4* x, double2* Y, double* part) {
   __shared__ double sh[32];
+  dep_wait();
+  dep_trigger();
   const int vol = (int)op.vol;
   const int64_t h = op.h;
   const int s = blockIdx.x * kDfSites + (threadIdx.x % kDfSites);
@@ -1104,10 +1107,11 @@ struct ChebConsts {
 // thread reads an entry before writing it); neighbours are read from x only.
 template <typename LinkT>
 __global__ void __launch_bounds__(3 * kDfSites, kDfMinBlocks)
-stencil_df_cheb_kernel(OpDev op, const float4* __restrict__ x, const float4* t_prev, float4* t_next,
-                       float4* __restrict__ acc, const float4* __restrict__ v, double2* __restrict__ y,
-                       double* __restrict__ part, ChebConsts k, int init, int last) {
+stencil_df_cheb_kernel(OpDev op, const float4* x, const float4* t_prev, float4* t_next, float4* acc, const float4* v,
+                       double2* y, double* part, ChebConsts k, int init, int last) {
   __shared__ double sh[32];
+  dep_wait();
+  dep_trigger();
   const int vol = (int)op.vol;
   const int64_t h = op.h;
   const int s = blockIdx.x * kDfSites + (threadIdx.x % kDfSites);
@@ -1265,11 +1269,8 @@ cudaError_t launch_gather_pairs_df(const void* V, int64_t n, const int* order, i
 int matvec_df_blocks(const OpDev& op) { return (int)((op.vol + kDfSites - 1) / kDfSites); }
 
 cudaError_t launch_matvec_df(const OpDev& op, const void* x, void* y, double* part, cudaStream_t s) {
-  if (op.links32)
-    stencil_df_kernel<float2><<<matvec_df_blocks(op), 3 * kDfSites, 0, s>>>(op, (const float4*)x, (double2*)y, part);
-  else
-    stencil_df_kernel<float4><<<matvec_df_blocks(op), 3 * kDfSites, 0, s>>>(op, (const float4*)x, (double2*)y, part);
-  return cudaGetLastError();
+  return launch_dep(op.links32 ? stencil_df_kernel<float2> : stencil_df_kernel<float4>, dim3(matvec_df_blocks(op)),
+                    3 * kDfSites, s, op, (const float4*)x, (double2*)y, part);
 }
 
 cudaError_t launch_matvec_df_cheb(const OpDev& op, const void* x, const void* t_prev, void* t_next, void* acc,
@@ -1277,15 +1278,9 @@ cudaError_t launch_matvec_df_cheb(const OpDev& op, const void* x, const void* t_
                                   double g, double g0, int init, int last, cudaStream_t s) {
   auto f = [](double d) { const float hi = (float)d; return ff{hi, (float)(d - (double)hi)}; };
   ChebConsts k{f(kappa), f(m0), f(c), f(sc), f(g), f(g0)};
-  if (op.links32)
-    stencil_df_cheb_kernel<float2><<<matvec_df_blocks(op), 3 * kDfSites, 0, s>>>(
-        op, (const float4*)x, (const float4*)t_prev, (float4*)t_next, (float4*)acc, (const float4*)v, (double2*)y,
-        part, k, init, last);
-  else
-    stencil_df_cheb_kernel<float4><<<matvec_df_blocks(op), 3 * kDfSites, 0, s>>>(
-        op, (const float4*)x, (const float4*)t_prev, (float4*)t_next, (float4*)acc, (const float4*)v, (double2*)y,
-        part, k, init, last);
-  return cudaGetLastError();
+  return launch_dep(op.links32 ? stencil_df_cheb_kernel<float2> : stencil_df_cheb_kernel<float4>,
+                    dim3(matvec_df_blocks(op)), 3 * kDfSites, s, op, (const float4*)x, (const float4*)t_prev,
+                    (float4*)t_next, (float4*)acc, (const float4*)v, (double2*)y, part, k, init, last);
 }
 
 cudaError_t launch_links_df(const void* in, void* out, int64_t vol, cudaStream_t s) {

@@ -548,8 +548,7 @@ __global__ void __launch_bounds__(kT) gsfx_normalize_kernel(GSArgs a) {
 // about 3,000 clocks).
 template <bool Cluster>
 __global__ void __launch_bounds__(kT, 1)
-gsfx_step_coop_kernel(GSArgs a, const double2* __restrict__ alpha_part, int n_alpha_part, int passes,
-                      double* __restrict__ nrm2) {
+gsfx_step_coop_kernel(GSArgs a, const double2* alpha_part, int n_alpha_part, int passes, double* nrm2) {
   namespace cg = cooperative_groups;
   auto sync_all = [] {
     if constexpr (Cluster) cg::this_cluster().sync();
@@ -569,6 +568,8 @@ gsfx_step_coop_kernel(GSArgs a, const double2* __restrict__ alpha_part, int n_al
   const int64_t p1 = min(p0 + (int64_t)a.rows_per_block, h);
   StepState* st = a.st;
   const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+  dep_wait();
+  dep_trigger();
   double tmax = 0.0;                                 // thread 0 of every block
   if (threadIdx.x == 0) tmax = a.st->tmax;
   const double ar = block_dsum((const double*)alpha_part, 2, n_alpha_part, sh);   // every block, the same order
@@ -799,17 +800,20 @@ cudaError_t launch_gs_step_coop<double>(const GSArgs& a, const double2* alpha_pa
   cfg.blockDim = dim3(kT);
   cfg.dynamicSmemBytes = fx_smem(a.m);
   cfg.stream = s;
-  cudaLaunchAttribute at{};
-  cfg.attrs = &at;
+  cudaLaunchAttribute at[2] = {};
+  cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (grid <= kClusterMax) {   // the portable cluster size; one cluster
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = grid;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  if (grid <= kClusterMax) {   // the portable cluster size; one cluster, set up while the product ends
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = grid;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelExC(&cfg, (const void*)gsfx_step_coop_kernel<true>, args);
   }
-  at.id = cudaLaunchAttributeCooperative;
-  at.val.cooperative = 1;
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
   return cudaLaunchKernelExC(&cfg, (const void*)gsfx_step_coop_kernel<false>, args);
 }
 

@@ -26,10 +26,11 @@ constexpr int kMvThreads = 256;
 
 template <typename R, int MODE>
 __global__ void __launch_bounds__(kMvThreads)
-stencil_kernel(OpDev op, const cplx<R>* __restrict__ X, cplx<R>* __restrict__ Y, double* __restrict__ part,
-               const int* __restrict__ cand, const double* __restrict__ lam, int64_t ldx) {
+stencil_kernel(OpDev op, const cplx<R>* X, cplx<R>* Y, double* part, const int* cand, const double* lam, int64_t ldx) {
   using C = cplx<R>;
   __shared__ double sh[32];
+  dep_wait();
+  dep_trigger();
   const int64_t vol = op.vol, h = op.h;
   const int64_t t = (int64_t)blockIdx.x * kMvThreads + threadIdx.x;
   const int col = blockIdx.y;
@@ -135,10 +136,11 @@ constexpr int kFxSites = 32, kFxWarps = 12;
 
 template <int MinBlocks>
 __global__ void __launch_bounds__(32 * kFxWarps, MinBlocks)
-stencil_fx_kernel(OpDev op, const fxc* __restrict__ X, const int* __restrict__ Kx, const double2* __restrict__ x64,
-                  double2* __restrict__ Y, double* __restrict__ part) {
+stencil_fx_kernel(OpDev op, const fxc* X, const int* Kx, const double2* x64, double2* Y, double* part) {
   __shared__ double sh[32];
   __shared__ double2 wsum[6][kFxSites];
+  dep_wait();
+  dep_trigger();
   const int vol = (int)op.vol;
   const int64_t h = op.h;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -243,9 +245,11 @@ constexpr int kSiteMinBlocks = 5;
 
 template <int MODE>
 __global__ void __launch_bounds__(kSiteThreads, kSiteMinBlocks)
-stencil_site_kernel(OpDev op, const float2* __restrict__ X, float2* __restrict__ Y, double* __restrict__ part,
-                    const int* __restrict__ cand, const double* __restrict__ lam, int64_t ldx) {
+stencil_site_kernel(OpDev op, const float2* X, float2* Y, double* part, const int* cand, const double* lam,
+                    int64_t ldx) {
   __shared__ double sh[32];
+  dep_wait();
+  dep_trigger();
   const int vol = (int)op.vol;
   const int64_t h = op.h;
   const int s = blockIdx.x * kSitesPerBlock + (threadIdx.x % kSitesPerBlock);
@@ -336,10 +340,11 @@ constexpr int kDenseRowsPerBlock = kMvThreads / 32;
 
 template <typename R, int MODE>
 __global__ void __launch_bounds__(kMvThreads)
-dense_kernel(OpDev op, const cplx<R>* __restrict__ X, cplx<R>* __restrict__ Y, double* __restrict__ part,
-             const int* __restrict__ cand, const double* __restrict__ lam, int64_t ldx) {
+dense_kernel(OpDev op, const cplx<R>* X, cplx<R>* Y, double* part, const int* cand, const double* lam, int64_t ldx) {
   using C = cplx<R>;
   __shared__ double sh[32];
+  dep_wait();
+  dep_trigger();
   const int64_t h = op.h;
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kDenseRowsPerBlock + (threadIdx.x >> 5);
@@ -391,15 +396,12 @@ template <typename R, int MODE>
 cudaError_t launch_mode(const OpDev& op, const cplx<R>* x, cplx<R>* y, double* part, const int* cand,
                         const double* lam, int ncand, int64_t ldx, int nblk, cudaStream_t s) {
   dim3 grid(nblk, MODE == MV_RESID ? ncand : 1);
-  if (op.kind == JTRLAN_STENCIL4D) {
-    if constexpr (sizeof(R) == sizeof(float))
-      stencil_site_kernel<MODE><<<grid, kSiteThreads, 0, s>>>(op, x, y, part, cand, lam, ldx);
-    else
-      stencil_kernel<R, MODE><<<grid, kMvThreads, 0, s>>>(op, x, y, part, cand, lam, ldx);
-  } else {
-    dense_kernel<R, MODE><<<grid, kMvThreads, 0, s>>>(op, x, y, part, cand, lam, ldx);
-  }
-  return cudaGetLastError();
+  auto launch = [&](auto kernel, int threads) {
+    return launch_dep(kernel, grid, threads, s, op, x, y, part, cand, lam, ldx);
+  };
+  if (op.kind != JTRLAN_STENCIL4D) return launch(dense_kernel<R, MODE>, kMvThreads);
+  if constexpr (sizeof(R) == sizeof(float)) return launch(stencil_site_kernel<MODE>, kSiteThreads);
+  else return launch(stencil_kernel<R, MODE>, kMvThreads);
 }
 
 }  // namespace
@@ -413,9 +415,8 @@ cudaError_t launch_matvec_fx(const OpDev& op, const void* X, const int* Kx, cons
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int nb = matvec_fx_blocks(op);
-  (nb <= nsm ? stencil_fx_kernel<1> : stencil_fx_kernel<2>)<<<nb, 32 * kFxWarps, 0, s>>>(
-      op, (const fxc*)X, Kx, (const double2*)x64, (double2*)Y, part);
-  return cudaGetLastError();
+  return launch_dep(nb <= nsm ? stencil_fx_kernel<1> : stencil_fx_kernel<2>, dim3(nb), 32 * kFxWarps, s, op,
+                    (const fxc*)X, Kx, (const double2*)x64, (double2*)Y, part);
 }
 
 cudaError_t launch_links_fx(const void* in, void* out, int64_t vol, const int* kfx, cudaStream_t s) {
