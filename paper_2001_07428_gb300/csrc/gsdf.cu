@@ -1009,13 +1009,8 @@ __device__ __forceinline__ void stencil_df_sums_biased(const OpDev& op, const fl
       cbias_accc(r.ws2, r.we2, cneg(wf), p1);    // -W(s)^* x1(s+mu)
       cbias_accc(r.ws2, r.we2, wb, m1);          // +W(s-mu)^H x1(s-mu)
     };
-    if constexpr (sizeof(LinkT) == sizeof(float2)) {
 #pragma unroll
-      for (int b = 0; b < 3; ++b) products(b);
-    } else {   // (hi, lo) links: unrolled, the operands of the three b spill at 80 registers
-#pragma unroll 1
-      for (int b = 0; b < 3; ++b) products(b);
-    }
+    for (int b = 0; b < 3; ++b) products(b);
   }
 #pragma unroll
   for (int q = 0; q < 2; ++q) {   // the high parts without their bias (exact)
@@ -1105,8 +1100,11 @@ struct ChebConsts {
 // 10.5 s, the same products and restarts); on the last step acc goes out in FP64 to y, with the
 // per-block partials of conj(v) y (the alpha of Algorithm 2).  t_next may alias t_prev (the same
 // thread reads an entry before writing it); neighbours are read from x only.
-template <typename LinkT>
-__global__ void __launch_bounds__(3 * kDfSites, kDfMinBlocks)
+//
+// Blocks of 32 sites, MinBlocks of them on an SM (which sets the registers); df_cheb_per_sm chooses.
+constexpr int kChebSites = 32;
+template <typename LinkT, int MinBlocks>
+__global__ void __launch_bounds__(3 * kChebSites, MinBlocks)
 stencil_df_cheb_kernel(OpDev op, const float4* x, const float4* t_prev, float4* t_next, float4* acc, const float4* v,
                        double2* y, double* part, ChebConsts k, int init, int last) {
   __shared__ double sh[32];
@@ -1114,8 +1112,8 @@ stencil_df_cheb_kernel(OpDev op, const float4* x, const float4* t_prev, float4* 
   dep_trigger();
   const int vol = (int)op.vol;
   const int64_t h = op.h;
-  const int s = blockIdx.x * kDfSites + (threadIdx.x % kDfSites);
-  const int a = threadIdx.x / kDfSites;
+  const int s = blockIdx.x * kChebSites + (threadIdx.x % kChebSites);
+  const int a = threadIdx.x / kChebSites;
   double c0 = 0.0, c1 = 0.0;
   if (s < vol) {
     DfSums r;
@@ -1273,14 +1271,39 @@ cudaError_t launch_matvec_df(const OpDev& op, const void* x, void* y, double* pa
                     3 * kDfSites, s, op, (const float4*)x, (double2*)y, part);
 }
 
+int matvec_df_cheb_blocks(const OpDev& op) { return (int)((op.vol + kChebSites - 1) / kChebSites); }
+
+// Blocks of the fused step resident on an SM.  complex64 links: eight fill a large lattice best (24^3 x 48:
+// 237 us a step; six 242, five 261; 64 sites by four 242).  With few blocks for an SM the limit also spreads
+// them: the launch otherwise gives some SMs twice the blocks of others (from four to seven an SM on average a
+// step costs as much as eight), and the wider registers of four keep more loads in flight.  us a step at
+// 8 | 4 blocks an SM, the average count before:
+//   0.8 (8^4): 6.4 | 5.8, 1.7: 7.9 | 7.4, 2.5: 9.3 | 11.2, 3.4: 9.8 | 11.4, 4.2: 15.9 | 11.6, 5.1: 16.1 | 13.8,
+//   5.9: 16.2 | 16.3, 8.4: 19.1 | 18.1, 10: 22.0 | 22.1, 17: 32.6 | 33.5
+// (hi, lo) links want 142 registers (five blocks: 128) for the three columns of a direction at once; us a
+// step with one column at a time (64 sites by four, 80 registers) | now:
+//   0.8: 9.1 | 6.2, 1.7: 9.3 | 8.3, 2.5: 11.6 | 10.2, 3.4: 11.8 | 10.2, 4.2: 19.4 | 12.7, 6.7: 19.7 | 18.2,
+//   10: 27.9 | 25.2, 17: 44.4 | 40.5, 136 (24^3 x 48): 305 | 288
+static int df_cheb_per_sm(const OpDev& op) {
+  int dev = 0, nsm = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t nb = matvec_df_cheb_blocks(op), sm = nsm;
+  if (op.links32) return nb <= 2 * sm || (nb > 4 * sm && nb <= 6 * sm) ? 4 : 8;
+  return nb <= 4 * sm ? 4 : 5;
+}
+
 cudaError_t launch_matvec_df_cheb(const OpDev& op, const void* x, const void* t_prev, void* t_next, void* acc,
                                   const void* v, void* y, double* part, double kappa, double m0, double c, double sc,
                                   double g, double g0, int init, int last, cudaStream_t s) {
   auto f = [](double d) { const float hi = (float)d; return ff{hi, (float)(d - (double)hi)}; };
   ChebConsts k{f(kappa), f(m0), f(c), f(sc), f(g), f(g0)};
-  return launch_dep(op.links32 ? stencil_df_cheb_kernel<float2> : stencil_df_cheb_kernel<float4>,
-                    dim3(matvec_df_blocks(op)), 3 * kDfSites, s, op, (const float4*)x, (const float4*)t_prev,
-                    (float4*)t_next, (float4*)acc, (const float4*)v, (double2*)y, part, k, init, last);
+  const int per_sm = df_cheb_per_sm(op);
+  auto kernel = op.links32 ? (per_sm == 4 ? stencil_df_cheb_kernel<float2, 4> : stencil_df_cheb_kernel<float2, 8>)
+                           : (per_sm == 4 ? stencil_df_cheb_kernel<float4, 4> : stencil_df_cheb_kernel<float4, 5>);
+  return launch_dep(kernel, dim3(matvec_df_cheb_blocks(op)), 3 * kChebSites, s, op, (const float4*)x,
+                    (const float4*)t_prev, (float4*)t_next, (float4*)acc, (const float4*)v, (double2*)y, part, k, init,
+                    last);
 }
 
 cudaError_t launch_links_df(const void* in, void* out, int64_t vol, cudaStream_t s) {

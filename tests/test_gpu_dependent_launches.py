@@ -19,7 +19,7 @@ def _lib():
 
 def _solver(kind, size, precision, **kw):
     from paper_2001_07428_gb300.solver import JTRLan
-    par = dict(nev=4, m=24, mwin=8, tol=1e-8, precision=precision, device="cuda:0", **kw)
+    par = dict(nev=4, m=20, mwin=8, tol=1e-8, precision=precision, device="cuda:0", **kw)
     if kind == "dense":
         A11, A12 = inputs.dense_jsym(size, 3)
         return JTRLan("dense", A11=A11, A12=A12, **par)
@@ -87,3 +87,20 @@ def test_filter_chain(dims, links, degree):
         assert c.cpu().numpy().tobytes() == want
         assert bool(torch.isfinite(torch.view_as_real(b)).all())
     s.close()
+
+
+@pytest.mark.parametrize("links", ["c64", "c128"])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (3, 3, 3, 3), (11, 9, 13, 7), (16, 16, 16, 5), (13, 13, 13, 13), (16, 16, 16, 8)])
+def test_filter_splits_against_fp64(dims, links):
+    """Each block split of the fused step against the FP64 filter.  A step's products are good to 2^-40 of
+    the sum of their magnitudes, which is below 100 half-widths of the window here, and the recurrence
+    carries a step's error on at most degree times."""
+    degree = 9
+    kw = dict(links_dtype=links, filter_final_coeffs=np.linspace(1.0, 0.1, degree + 1), filter_window=(1.3, 18.7))
+    out = []
+    for precision in ("fp64", "mixed_reorth"):
+        s = _solver("stencil", dims, precision, **kw)
+        v = torch.from_numpy(inputs.random_vector(s.n, 7)).to("cuda:0")
+        out.append(s.apply_filter(v).cpu().numpy())
+        s.close()
+    assert np.abs(out[1] - out[0]).max() <= degree ** 2 * 100 * 2.0 ** -40 * np.abs(out[0]).max()
