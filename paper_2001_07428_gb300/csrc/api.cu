@@ -106,7 +106,8 @@ struct Phase {
   size_t cs = 0;          // bytes per complex number of V
   double* alpha_part = nullptr;
   double* resid_part = nullptr;
-  int mv_nblk = 0;
+  int mv_nblk = 0;      // blocks of a residual product
+  int alpha_nblk = 0;   // partials of x^H y of a product
   int which = JTRLAN_SMALLEST;  // the wanted end of this phase's operator
   bool filtered = false;        // the Lanczos product is B = p(A)
   bool certify = false;         // filtered phase judged by the true residual of A at x^H A x
@@ -292,7 +293,7 @@ jtrlan_status setup_certify(jtrlan_ctx* c, const double* coeffs, int degree) {
     for (int b = 0; b < 3; ++b) JT_TRY(c->dalloc(&ph.fbuf[b], (size_t)c->n * sizeof(double2)));
     JT_TRY(c->dalloc(&ph.fbuf[3], (size_t)c->n * sizeof(float4)));
     const int nb = std::max(cheb_blocks(c->n), ph.dfmv ? std::max(matvec_df_blocks(ph.opdf), matvec_df_cheb_blocks(ph.opdf))
-                                                       : ph.mv_nblk);
+                                                       : ph.alpha_nblk);
     JT_TRY(c->dalloc(&ph.alpha_part, (size_t)nb * sizeof(double2)));
     JT_TRY(c->dalloc(&ph.resid_part, (size_t)std::max(nb, ph.mv_nblk * c->nev) * sizeof(double)));
   }
@@ -343,10 +344,11 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
   auto make_phase = [&](Phase& ph, size_t cs) -> jtrlan_status {
     ph.cs = cs;
     ph.mv_nblk = matvec_blocks(ph.op);
+    ph.alpha_nblk = matvec_alpha_blocks(ph.op);
     JT_TRY(c->dalloc(&ph.V, (size_t)c->n * (m + 1) * cs));
     JT_TRY(c->dalloc(&ph.Vtmp, (size_t)c->n * std::max(c->kk, 1) * cs));
     JT_TRY(c->dalloc(&ph.y, (size_t)c->n * cs));
-    JT_TRY(c->dalloc(&ph.alpha_part, (size_t)ph.mv_nblk * sizeof(double2)));
+    JT_TRY(c->dalloc(&ph.alpha_part, (size_t)ph.alpha_nblk * sizeof(double2)));
     JT_TRY(c->dalloc(&ph.resid_part, (size_t)ph.mv_nblk * c->nev * sizeof(double)));
     return JTRLAN_OK;
   };
@@ -374,7 +376,7 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
       } else {
         cudaGetLastError();
       }
-      if (c->p64.fxmv && matvec_fx_blocks(d) > c->p64.mv_nblk)
+      if (c->p64.fxmv && matvec_fx_blocks(d) > c->p64.alpha_nblk)
         JT_TRY(c->dalloc(&c->p64.alpha_part, (size_t)matvec_fx_blocks(d) * sizeof(double2)));
     }
   } else {  // double-float phase on the FP64 operator
@@ -399,7 +401,7 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
       }
       c->pdf.dfmv = true;
       const int nb = matvec_df_blocks(d);
-      if (nb > c->pdf.mv_nblk) JT_TRY(c->dalloc(&c->pdf.alpha_part, (size_t)nb * sizeof(double2)));
+      if (nb > c->pdf.alpha_nblk) JT_TRY(c->dalloc(&c->pdf.alpha_part, (size_t)nb * sizeof(double2)));
     }
   }
   if (c->mixed && !prm->rotate_simt && m <= tc_rotate_max_m()) {   // restart rotation on the tensor cores
@@ -441,11 +443,12 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
         c->p32.which = JTRLAN_LARGEST;
         c->p32.fcoef.assign(prm->filter_coeffs, prm->filter_coeffs + prm->filter_degree + 1);
         for (int b = 0; b < 3; ++b) JT_TRY(c->dalloc(&c->p32.fbuf[b], (size_t)c->n * sizeof(float2)));
-        if (cheb_blocks(c->n) > c->p32.mv_nblk)
+        if (cheb_blocks(c->n) > c->p32.alpha_nblk)
           JT_TRY(c->dalloc(&c->p32.alpha_part, (size_t)cheb_blocks(c->n) * sizeof(double2)));
       }
     } else {
       c->p32.mv_nblk = matvec_blocks(q);
+      c->p32.alpha_nblk = matvec_alpha_blocks(q);
     }
   }
   c->p64.which = c->pdf.which = prm->which;
@@ -457,11 +460,11 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
     JT_TRY(c->dalloc(&c->cg_p, (size_t)c->n * sizeof(double2)));
     JT_TRY(c->dalloc(&c->cg_q, (size_t)c->n * sizeof(double2)));
     JT_TRY(c->dalloc(&c->cg_part, (size_t)cg_blocks(c->n) * sizeof(double)));
-    JT_TRY(c->dalloc(&c->cg_pq, (size_t)c->p64.mv_nblk * sizeof(double2)));
+    JT_TRY(c->dalloc(&c->cg_pq, (size_t)c->p64.alpha_nblk * sizeof(double2)));
     JT_TRY(c->dalloc(&c->cg_st, sizeof(CgState)));
     JT_TRY(c->halloc(&c->h_cgst, sizeof(CgState)));
     JT_CUDA(cudaMemsetAsync(c->cg_st, 0, sizeof(CgState), c->stream));
-    if (cg_blocks(c->n) > c->p64.mv_nblk)
+    if (cg_blocks(c->n) > c->p64.alpha_nblk)
       JT_TRY(c->dalloc(&c->p64.alpha_part, (size_t)cg_blocks(c->n) * sizeof(double2)));
     if (cg_blocks(c->n) > c->p64.mv_nblk * c->nev)
       JT_TRY(c->dalloc(&c->p64.resid_part, (size_t)cg_blocks(c->n) * sizeof(double)));
@@ -661,7 +664,7 @@ jtrlan_status rq_resid(jtrlan_ctx* c, Phase& ph, const void* x, double* lam_out,
   } else {
     LAUNCH(K_RESID, launch_matvec<double>(ph.op, (const double2*)x, (double2*)ph.fbuf[0], MV_ALPHA, ph.alpha_part,
                                           nullptr, nullptr, 0, 0, nullptr, s));
-    nparts = ph.mv_nblk;
+    nparts = ph.alpha_nblk;
   }
   LAUNCH(K_RESID, launch_sum_re(ph.alpha_part, nparts, lam_out, s));
   LAUNCH(K_RESID, launch_resid_part(ph.fbuf[0], x, lam_out, n, ph.resid_part, s));
@@ -683,7 +686,7 @@ jtrlan_status cg_solve(jtrlan_ctx* c, Phase& ph, const void* b, void* y) {
     for (int u = 0; u < kCgGroup; ++u) {
       cudaError_t e = launch_matvec<double>(ph.op, (const double2*)c->cg_p, (double2*)c->cg_q, MV_ALPHA, c->cg_pq,
                                             nullptr, nullptr, 0, 0, nullptr, st);
-      if (e == cudaSuccess) e = launch_cg_alpha(c->cg_pq, ph.mv_nblk, c->cg_st, st);
+      if (e == cudaSuccess) e = launch_cg_alpha(c->cg_pq, ph.alpha_nblk, c->cg_st, st);
       if (e == cudaSuccess) e = launch_cg_update(y, c->cg_r, c->cg_p, c->cg_q, n, c->cg_part, c->cg_st, st);
       if (e != cudaSuccess) return e;
     }
@@ -719,7 +722,7 @@ jtrlan_status cg_solve(jtrlan_ctx* c, Phase& ph, const void* b, void* y) {
       for (int u = 0; u < kCgGroup; ++u) {
         LAUNCH(K_CG, launch_matvec<double>(ph.op, (const double2*)c->cg_p, (double2*)c->cg_q, MV_ALPHA, c->cg_pq,
                                            nullptr, nullptr, 0, 0, nullptr, s));
-        LAUNCH(K_CG, launch_cg_alpha(c->cg_pq, ph.mv_nblk, c->cg_st, s));
+        LAUNCH(K_CG, launch_cg_alpha(c->cg_pq, ph.alpha_nblk, c->cg_st, s));
         LAUNCH(K_CG, launch_cg_update(y, c->cg_r, c->cg_p, c->cg_q, n, c->cg_part, c->cg_st, s));
         c->nl[K_CG] += 2;   // three kernels
       }
@@ -758,7 +761,7 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
   const int mv_parts = c->invert ? cg_blocks(n)
                        : (filtered && !(ph.certify && ph.dfmv)) ? cheb_blocks(n)
                        : ph.dfmv ? (filtered ? matvec_df_cheb_blocks(ph.opdf) : matvec_df_blocks(ph.opdf))
-                       : ph.fxmv && !filtered ? matvec_fx_blocks(ph.opfx) : ph.mv_nblk;
+                       : ph.fxmv && !filtered ? matvec_fx_blocks(ph.opfx) : ph.alpha_nblk;
   for (int j = j0; j < j1; ++j) {
     if (filtered) {
       if constexpr (std::is_same<R, float>::value)

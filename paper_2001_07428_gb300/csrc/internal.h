@@ -35,7 +35,7 @@ struct OpDev {
 // Modes of the matvec kernels.
 enum MvMode { MV_PLAIN = 0, MV_ALPHA = 1, MV_RESID = 2 };
 
-// y = A x.  MV_ALPHA also writes per-block partial sums of x^H y to part (double2[nblk]).
+// y = A x.  MV_ALPHA also writes per-block partial sums of x^H y to part (double2[matvec_alpha_blocks]).
 // MV_RESID takes ncand columns x_c = X[:, cand[c]] (ld = n), computes ||A x_c - lam[c] x_c||^2
 // per block into part[c * nblk + b] (double) and writes no y.  Returns the per-column block
 // count (nblk) through *nblk_out.
@@ -43,7 +43,8 @@ template <typename R>
 cudaError_t launch_matvec(const OpDev& op, const cplx<R>* x, cplx<R>* y, MvMode mode, double* part,
                           const int* cand, const double* lam, int ncand, int64_t ldx,
                           int* nblk_out, cudaStream_t s);
-int matvec_blocks(const OpDev& op);  // nblk of launch_matvec for one column
+int matvec_blocks(const OpDev& op);        // nblk of launch_matvec for one column (MV_RESID)
+int matvec_alpha_blocks(const OpDev& op);  // partials of MV_ALPHA
 // FP64 stencil product by integer sums (matvec.cu): y = A x for x as fixed point (X on *Kx) and in FP64
 // (x64), fixed-point links in op; part: matvec_fx_blocks double2 partials of x^H y.
 int matvec_fx_blocks(const OpDev& op);

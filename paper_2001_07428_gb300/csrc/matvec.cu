@@ -392,6 +392,68 @@ dense_kernel(OpDev op, const cplx<R>* X, cplx<R>* Y, double* part, const int* ca
   }
 }
 
+// Dense with fewer rows than fill the chip at eight a block: a block of four warps a row, one on each of the
+// SM's quarters.  An FP64 instruction holds its quarter's pipe for 64 clocks, so the kernel above, at two rows
+// a quarter and four sums of 32 lanes each, is a chain of pipe slots on h / 8 SMs.  us a product, eight rows a
+// block against one:  h = 40: 11.9 / 6.4, 100: 16.0 / 6.7, 304: 20.9 / 9.8, 608: 29.2 / 16.7, 1000: 46.3 / 39.2,
+// 1216: 49.5 / 47.1.
+// The four sums of a warp end as one value on every eighth lane (6 additions a lane instead of 20).
+constexpr int kRowWarps = 4;
+
+template <typename R, int MODE>
+__global__ void __launch_bounds__(32 * kRowWarps)
+dense_row_kernel(OpDev op, const cplx<R>* x, cplx<R>* Y, double* part) {
+  using C = cplx<R>;
+  __shared__ double sums[kRowWarps][4];
+  dep_wait();
+  dep_trigger();
+  const int64_t h = op.h, row = blockIdx.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const C* r11 = (const C*)op.a11 + row * h;
+  const C* r12 = (const C*)op.a12 + row * h;
+  C y1 = mk<R>(0, 0), y2 = mk<R>(0, 0);
+  for (int64_t c = threadIdx.x; c < h; c += 32 * kRowWarps) {
+    const C a11 = r11[c], a12 = r12[c], x1 = x[c], x2 = x[h + c];
+    y1 = cfma(a11, x1, y1);
+    y1 = cfma(a12, x2, y1);
+    y2 = cfmac(a11, x2, y2);
+    y2 = cfmac(mk<R>(-a12.x, -a12.y), x1, y2);
+  }
+  const bool up = lane & 16, odd = lane & 8;
+  double p = (double)(up ? y2.x : y1.x), q = (double)(up ? y2.y : y1.y);
+  p += __shfl_xor_sync(0xffffffffu, (double)(up ? y1.x : y2.x), 16);
+  q += __shfl_xor_sync(0xffffffffu, (double)(up ? y1.y : y2.y), 16);
+  double v = (odd ? q : p) + __shfl_xor_sync(0xffffffffu, odd ? p : q, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((lane & 7) == 0) sums[w][lane >> 3] = v;
+  __syncthreads();
+  if (w == 0) {
+    const double* t = &sums[0][lane & 3];
+    const double s = (t[0] + t[4]) + (t[8] + t[12]);
+    const double s0 = __shfl_sync(0xffffffffu, s, 0), s1 = __shfl_sync(0xffffffffu, s, 1);
+    const double s2 = __shfl_sync(0xffffffffu, s, 2), s3 = __shfl_sync(0xffffffffu, s, 3);
+    const C o1 = mk<R>((R)s0, (R)s1), o2 = mk<R>((R)s2, (R)s3);
+    if (lane < 2) {
+      Y[lane ? h + row : row] = lane ? o2 : o1;
+      if (MODE == MV_ALPHA) {   // lane 0: Re(conj(x) y), lane 1: Im
+        const C x1 = x[row], x2 = x[h + row];
+        const double a = lane ? -(double)x1.y : (double)x1.x, b = lane ? (double)x1.x : (double)x1.y;
+        const double c = lane ? -(double)x2.y : (double)x2.x, d = lane ? (double)x2.x : (double)x2.y;
+        part[2 * row + lane] = a * o1.x + b * o1.y + c * o2.x + d * o2.y;
+      }
+    }
+  }
+}
+
+// Rows taken one a block: as long as eight a block would leave SMs without one.
+bool dense_by_row(const OpDev& op) {
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  return op.kind != JTRLAN_STENCIL4D && op.h <= (int64_t)kDenseRowsPerBlock * nsm;
+}
+
 template <typename R, int MODE>
 cudaError_t launch_mode(const OpDev& op, const cplx<R>* x, cplx<R>* y, double* part, const int* cand,
                         const double* lam, int ncand, int64_t ldx, int nblk, cudaStream_t s) {
@@ -399,6 +461,9 @@ cudaError_t launch_mode(const OpDev& op, const cplx<R>* x, cplx<R>* y, double* p
   auto launch = [&](auto kernel, int threads) {
     return launch_dep(kernel, grid, threads, s, op, x, y, part, cand, lam, ldx);
   };
+  if constexpr (MODE != MV_RESID)
+    if (dense_by_row(op))
+      return launch_dep(dense_row_kernel<R, MODE>, dim3((unsigned)op.h), 32 * kRowWarps, s, op, x, y, part);
   if (op.kind != JTRLAN_STENCIL4D) return launch(dense_kernel<R, MODE>, kMvThreads);
   if constexpr (sizeof(R) == sizeof(float)) return launch(stencil_site_kernel<MODE>, kSiteThreads);
   else return launch(stencil_kernel<R, MODE>, kMvThreads);
@@ -431,6 +496,7 @@ int matvec_blocks(const OpDev& op) {
   }
   return (int)((op.h + kDenseRowsPerBlock - 1) / kDenseRowsPerBlock);
 }
+int matvec_alpha_blocks(const OpDev& op) { return dense_by_row(op) ? (int)op.h : matvec_blocks(op); }
 
 template <typename R>
 cudaError_t launch_matvec(const OpDev& op, const cplx<R>* x, cplx<R>* y, MvMode mode, double* part,
