@@ -89,9 +89,9 @@ BYTES_PER_UNIT = {"matvec": 84 * 16.0, "resid": 84 * 16.0, "gs_first": 32.0, "gs
 # SHA-256 of the source file the capture was built from: the figure is reported only while that file
 # is unchanged (roofline.traffic is null otherwise).
 NCU_TRAFFIC = {
-    "matvec": dict(bytes=688.0e6, workload="stencil_24x24x24x48", kernel="stencil_df_cheb_kernel<float2, 8> (middle step)",
+    "matvec": dict(bytes=688.4e6, workload="stencil_24x24x24x48", kernel="stencil_df_cheb_kernel<float2, 32, 8> (middle step)",
                    source="paper_2001_07428_gb300/csrc/gsdf.cu",
-                   sha256="53a3c4f57543eb879987187ac515f9fa1b4c184400c1a57949930f92d778d3cb"),
+                   sha256="c2b0951ee48049b03517a8577d49fbe4bbc4e41aec573dd88ab9d5cefbc4c298"),
     "gs_step": dict(bytes=13.66e6, workload="stencil_8x8x8x8", kernel="gs_step_coop_kernel<double>",
                     source="paper_2001_07428_gb300/csrc/gs.cu",
                     sha256="25f4b188216fe6b311d90026b3e55046646e3a430ba0d7a2b9d8b809fdae98b5"),

@@ -292,8 +292,7 @@ jtrlan_status setup_certify(jtrlan_ctx* c, const double* coeffs, int degree) {
     ph.which = JTRLAN_LARGEST;
     for (int b = 0; b < 3; ++b) JT_TRY(c->dalloc(&ph.fbuf[b], (size_t)c->n * sizeof(double2)));
     JT_TRY(c->dalloc(&ph.fbuf[3], (size_t)c->n * sizeof(float4)));
-    const int nb = std::max(cheb_blocks(c->n), ph.dfmv ? std::max(matvec_df_blocks(ph.opdf), matvec_df_cheb_blocks(ph.opdf))
-                                                       : ph.alpha_nblk);
+    const int nb = std::max(cheb_blocks(c->n), ph.dfmv ? matvec_df_blocks(ph.opdf) : ph.alpha_nblk);
     JT_TRY(c->dalloc(&ph.alpha_part, (size_t)nb * sizeof(double2)));
     JT_TRY(c->dalloc(&ph.resid_part, (size_t)std::max(nb, ph.mv_nblk * c->nev) * sizeof(double)));
   }
@@ -760,7 +759,7 @@ jtrlan_status lanczos_steps(jtrlan_ctx* c, Phase& ph, GSArgs& a, int j0, int j1,
   if (ph.fx) LAUNCH(K_OTHER, launch_load_col(ph.V, c->vexp, n, j0, (double2*)ph.x, s));
   const int mv_parts = c->invert ? cg_blocks(n)
                        : (filtered && !(ph.certify && ph.dfmv)) ? cheb_blocks(n)
-                       : ph.dfmv ? (filtered ? matvec_df_cheb_blocks(ph.opdf) : matvec_df_blocks(ph.opdf))
+                       : ph.dfmv ? matvec_df_blocks(ph.opdf)
                        : ph.fxmv && !filtered ? matvec_fx_blocks(ph.opfx) : ph.alpha_nblk;
   for (int j = j0; j < j1; ++j) {
     if (filtered) {

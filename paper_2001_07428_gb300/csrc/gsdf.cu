@@ -1101,10 +1101,12 @@ struct ChebConsts {
 // per-block partials of conj(v) y (the alpha of Algorithm 2).  t_next may alias t_prev (the same
 // thread reads an entry before writing it); neighbours are read from x only.
 //
-// Blocks of 32 sites, MinBlocks of them on an SM (which sets the registers); df_cheb_per_sm chooses.
+// Blocks of Sites sites, MinBlocks of them on an SM (which sets the registers): 32 sites and
+// df_cheb_per_sm's choice, but on the last step the blocks of the Dot2 product, so that the partials of
+// alpha, their count and order, do not depend on the split.
 constexpr int kChebSites = 32;
-template <typename LinkT, int MinBlocks>
-__global__ void __launch_bounds__(3 * kChebSites, MinBlocks)
+template <typename LinkT, int Sites, int MinBlocks>
+__global__ void __launch_bounds__(3 * Sites, MinBlocks)
 stencil_df_cheb_kernel(OpDev op, const float4* x, const float4* t_prev, float4* t_next, float4* acc, const float4* v,
                        double2* y, double* part, ChebConsts k, int init, int last) {
   __shared__ double sh[32];
@@ -1112,8 +1114,8 @@ stencil_df_cheb_kernel(OpDev op, const float4* x, const float4* t_prev, float4* 
   dep_trigger();
   const int vol = (int)op.vol;
   const int64_t h = op.h;
-  const int s = blockIdx.x * kChebSites + (threadIdx.x % kChebSites);
-  const int a = threadIdx.x / kChebSites;
+  const int s = blockIdx.x * Sites + (threadIdx.x % Sites);
+  const int a = threadIdx.x / Sites;
   double c0 = 0.0, c1 = 0.0;
   if (s < vol) {
     DfSums r;
@@ -1271,7 +1273,7 @@ cudaError_t launch_matvec_df(const OpDev& op, const void* x, void* y, double* pa
                     3 * kDfSites, s, op, (const float4*)x, (double2*)y, part);
 }
 
-int matvec_df_cheb_blocks(const OpDev& op) { return (int)((op.vol + kChebSites - 1) / kChebSites); }
+static int df_cheb_blocks(const OpDev& op) { return (int)((op.vol + kChebSites - 1) / kChebSites); }
 
 // Blocks of the fused step resident on an SM.  complex64 links: eight fill a large lattice best (24^3 x 48:
 // 237 us a step; six 242, five 261; 64 sites by four 242).  With few blocks for an SM the limit also spreads
@@ -1288,7 +1290,7 @@ static int df_cheb_per_sm(const OpDev& op) {
   int dev = 0, nsm = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t nb = matvec_df_cheb_blocks(op), sm = nsm;
+  const int64_t nb = df_cheb_blocks(op), sm = nsm;
   if (op.links32) return nb <= 2 * sm || (nb > 4 * sm && nb <= 6 * sm) ? 4 : 8;
   return nb <= 4 * sm ? 4 : 5;
 }
@@ -1298,12 +1300,17 @@ cudaError_t launch_matvec_df_cheb(const OpDev& op, const void* x, const void* t_
                                   double g, double g0, int init, int last, cudaStream_t s) {
   auto f = [](double d) { const float hi = (float)d; return ff{hi, (float)(d - (double)hi)}; };
   ChebConsts k{f(kappa), f(m0), f(c), f(sc), f(g), f(g0)};
-  const int per_sm = df_cheb_per_sm(op);
-  auto kernel = op.links32 ? (per_sm == 4 ? stencil_df_cheb_kernel<float2, 4> : stencil_df_cheb_kernel<float2, 8>)
-                           : (per_sm == 4 ? stencil_df_cheb_kernel<float4, 4> : stencil_df_cheb_kernel<float4, 5>);
-  return launch_dep(kernel, dim3(matvec_df_cheb_blocks(op)), 3 * kChebSites, s, op, (const float4*)x,
-                    (const float4*)t_prev, (float4*)t_next, (float4*)acc, (const float4*)v, (double2*)y, part, k, init,
-                    last);
+  auto launch = [&](auto kernel, int blocks, int sites) {
+    return launch_dep(kernel, dim3(blocks), 3 * sites, s, op, (const float4*)x, (const float4*)t_prev, (float4*)t_next,
+                      (float4*)acc, (const float4*)v, (double2*)y, part, k, init, last);
+  };
+  if (last)
+    return launch(op.links32 ? stencil_df_cheb_kernel<float2, kDfSites, 4> : stencil_df_cheb_kernel<float4, kDfSites, 2>,
+                  matvec_df_blocks(op), kDfSites);
+  const bool four = df_cheb_per_sm(op) == 4;
+  return launch(op.links32 ? (four ? stencil_df_cheb_kernel<float2, kChebSites, 4> : stencil_df_cheb_kernel<float2, kChebSites, 8>)
+                           : (four ? stencil_df_cheb_kernel<float4, kChebSites, 4> : stencil_df_cheb_kernel<float4, kChebSites, 5>),
+                df_cheb_blocks(op), kChebSites);
 }
 
 cudaError_t launch_links_df(const void* in, void* out, int64_t vol, cudaStream_t s) {

@@ -163,8 +163,7 @@ cudaError_t launch_matvec_df(const OpDev& op, const void* x, void* y, double* pa
 // One Chebyshev step of B = p(A) fused into the compensated-FP32 stencil product (x, t_prev, t_next,
 // acc, v: (hi, lo) float4 vectors; t_next may alias t_prev): t_next = sc (A x - c x) - t_prev,
 // acc = g0 v + g t_next (init) or acc += g t_next; on the last step acc goes to y (FP64) with
-// matvec_df_cheb_blocks(op) double2 partials of conj(v) y in part.
-int matvec_df_cheb_blocks(const OpDev& op);
+// matvec_df_blocks(op) double2 partials of conj(v) y in part.
 cudaError_t launch_matvec_df_cheb(const OpDev& op, const void* x, const void* t_prev, void* t_next, void* acc,
                                   const void* v, void* y, double* part, double kappa, double m0, double c, double sc,
                                   double g, double g0, int init, int last, cudaStream_t s);
@@ -248,7 +247,7 @@ struct BatchArgs {
   const int64_t* vec_off;
   long long* prof;
   int* queue;
-  int mv_rows;     // tile: rows of the product a warp takes at once (1 or 2; they share the loads of x)
+  int mv_rows;     // tile of the compensated form: rows of the product a warp takes at once (1 or 2)
   int gs_groups;   // tile: most thread groups splitting the columns of the compensated update (0: all that fit)
 };
 constexpr int kBatchStats = 6;
