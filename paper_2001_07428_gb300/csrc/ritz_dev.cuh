@@ -30,34 +30,49 @@ struct TbarView {
   __device__ __forceinline__ double off(int j) const { return T[(size_t)(j + 1) * ld + j]; } // j >= k
 };
 
-template <typename F>
-__device__ __noinline__ int inertia(const TbarView& t, F sigma, F pivmin) {
+// The count in FP32, for the multisection: d the diagonal, b2 the squares of the arrow (i < k) and of the
+// off-diagonals (b2[j] of t_{j,j+1}, j >= k).  The quotients are the fast ones, good to 2 ulp, which the
+// slack of the bracket covers.
+__device__ __noinline__ int inertia32(const float* d, const float* b2, int k, int m, float sigma, float pivmin) {
   int neg = 0;
-  F s = 0;
-  for (int i = 0; i < t.k; ++i) {
-    F p = (F)t.diag(i) - sigma;
-    if (fabs(p) < pivmin) p = -pivmin;
-    neg += p < 0;
-    const F b = (F)t.arrow(i);
-    s += b * b / p;
+  float s = 0.f;
+  for (int i = 0; i < k; ++i) {
+    float p = d[i] - sigma;
+    if (fabsf(p) < pivmin) p = -pivmin;
+    neg += p < 0.f;
+    s += __fdividef(b2[i], p);
   }
-  F p = (F)t.diag(t.k) - sigma - s;
-  if (fabs(p) < pivmin) p = -pivmin;
-  neg += p < 0;
-  for (int j = t.k + 1; j < t.m; ++j) {
-    const F b = (F)t.off(j - 1);
-    p = (F)t.diag(j) - sigma - b * b / p;
-    if (fabs(p) < pivmin) p = -pivmin;
-    neg += p < 0;
+  float p = d[k] - sigma - s;
+  if (fabsf(p) < pivmin) p = -pivmin;
+  neg += p < 0.f;
+  for (int j = k + 1; j < m; ++j) {
+    p = d[j] - sigma - __fdividef(b2[j - 1], p);
+    if (fabsf(p) < pivmin) p = -pivmin;
+    neg += p < 0.f;
   }
   return neg;
 }
 
+// The tridiagonal part k .. m - 1 is eliminated from both ends at once, by two lanes: one takes k .. c
+// forward, the other m - 1 .. c + 1 backward, and the last pivot joins them.  An FP64 instruction holds its
+// pipe for 64 clocks whatever the active lanes, and this chain (a division an index) is most of a Ritz pair's
+// time: a restart at m = 30 (this and its verification) went from 143 to 84 us with both ends at once, the two
+// verification counts in one pass and FP32 copies for the multisection.
+struct TwoEnds {
+  int l, cnt, nf;        // this lane's end, its count, the longer (forward) count
+  int j, dj;             // its first index and direction
+  __device__ __forceinline__ TwoEnds(int k, int m, int end) : l(end) {
+    nf = (m - k + 1) / 2;
+    cnt = end ? m - k - nf : nf;
+    j = end ? m - 1 : k;
+    dj = end ? -1 : 1;
+  }
+};
+
 // Warp-cooperative solve of (T - sigma I) x = z in place (z: right-hand side on entry, in shared
 // memory); ipiv receives the reciprocal pivots.  The k eliminations of the diagonal part are
-// independent and run across the lanes; the tridiagonal part is a serial chain on lane 0.  On this
-// part one FP64 warp instruction holds the FP64 pipe for ~16 cycles whatever the active mask, so
-// the serial chain does one division per index and multiplies by stored reciprocals elsewhere.
+// independent and run across the lanes; the tridiagonal part goes on lanes 0 and 1, with one division an
+// index and stored reciprocals elsewhere.
 __device__ __noinline__ void shifted_solve_warp(const TbarView& t, double sigma, double pivmin, double* z, double* ipiv) {
   const int k = t.k, m = t.m, lane = threadIdx.x & 31;
   double s = 0.0, sr = 0.0;
@@ -72,27 +87,48 @@ __device__ __noinline__ void shifted_solve_warp(const TbarView& t, double sigma,
   }
   s = warp_sum(s);
   sr = warp_sum(sr);
-  if (lane == 0) {
-    double p = t.diag(k) - sigma - s;
-    if (fabs(p) < pivmin) p = (p < 0 ? -pivmin : pivmin);
-    double ip = 1.0 / p;
-    ipiv[k] = ip;
-    double zp = z[k] - sr;
-    z[k] = zp;
-    for (int j = k + 1; j < m; ++j) {
-      const double b = t.off(j - 1);
+  if (lane < 2) {
+    const TwoEnds e(k, m, lane);
+    double ip = 0.0, zp = 0.0, b = 0.0;   // of the index before; b couples the two
+    int j = e.j;
+    for (int i = 0; i < e.cnt; ++i, j += e.dj) {
       const double l = b * ip;
       double q = t.diag(j) - sigma - b * l;
-      if (fabs(q) < pivmin) q = (q < 0 ? -pivmin : pivmin);
-      ip = 1.0 / q;
-      ipiv[j] = ip;
       zp = z[j] - l * zp;
+      if (i == 0 && !e.l) {
+        q -= s;
+        zp -= sr;
+      }
       z[j] = zp;
+      const int c = e.l ? j - 1 : j;                       // the coupling to the next index, or across the middle
+      if (c >= k && c + 1 < m) b = t.off(c);
+      if (i + 1 < e.cnt || !e.l) {                         // the backward end's last pivot is the joined one
+        if (fabs(q) < pivmin) q = (q < 0 ? -pivmin : pivmin);
+        ip = 1.0 / q;
+        ipiv[j] = ip;
+      } else {
+        ip = q;                                            // carried to the join
+      }
     }
-    double zn = z[m - 1] * ipiv[m - 1];
-    z[m - 1] = zn;
-    for (int j = m - 2; j >= k; --j) {
-      zn = (z[j] - t.off(j) * zn) * ipiv[j];
+    // join: x_{c+1} = (z_{c+1} - b z_c / q_c) / (q_{c+1} - b^2 / q_c), x_c = (z_c - b x_{c+1}) / q_c
+    const double ipc = __shfl_sync(3u, ip, 0), zc = __shfl_sync(3u, zp, 0), bc = __shfl_sync(3u, b, 0);
+    const double qe = __shfl_sync(3u, ip, 1), ze = __shfl_sync(3u, zp, 1);
+    double zn;
+    if (m - k > 1) {
+      const double l = bc * ipc;
+      double q = qe - bc * l;
+      if (fabs(q) < pivmin) q = (q < 0 ? -pivmin : pivmin);
+      const double xe = (ze - l * zc) / q;
+      zn = lane ? xe : (zc - bc * xe) * ipc;
+    } else {
+      zn = zc * ipc;
+    }
+    j -= e.dj;                                             // this end's last index
+    if (e.cnt > 0) z[j] = zn;
+    for (int i = 1; i < e.cnt; ++i) {
+      const double o = t.off(e.l ? j : j - 1);
+      j -= e.dj;
+      zn = (z[j] - o * zn) * ipiv[j];
       z[j] = zn;
     }
   }
@@ -102,33 +138,51 @@ __device__ __noinline__ void shifted_solve_warp(const TbarView& t, double sigma,
   __syncwarp();
 }
 
-// Warp-cooperative FP64 inertia count of T - sigma I (same elimination order as above).
-__device__ int inertia_warp(const TbarView& t, double sigma, double pivmin) {
-  const int k = t.k, m = t.m, lane = threadIdx.x & 31;
+// Warp-cooperative FP64 inertia counts of T - sigma I for two shifts (lanes 0 .. 15 and 16 .. 31 take one
+// each), the elimination as above.  Lane 0 returns the count of s0 and lane 16 that of s1.
+__device__ __noinline__ int inertia2_warp(const TbarView& t, double s0, double s1, double pivmin) {
+  const int k = t.k, m = t.m, lane = threadIdx.x & 31, sub = lane & 15;
+  const double sigma = lane < 16 ? s0 : s1;
   double s = 0.0;
   int neg = 0;
-  for (int i = lane; i < k; i += 32) {
+  for (int i = sub; i < k; i += 16) {
     double p = t.diag(i) - sigma;
     if (fabs(p) < pivmin) p = -pivmin;
     neg += p < 0;
     const double b = t.arrow(i);
     s += b * b / p;
   }
-  s = warp_sum(s);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) neg += __shfl_xor_sync(0xffffffffu, neg, o);
-  if (lane == 0) {
-    double p = t.diag(k) - sigma - s;
-    if (fabs(p) < pivmin) p = -pivmin;
-    neg += p < 0;
-    for (int j = k + 1; j < m; ++j) {
-      const double b = t.off(j - 1);
-      p = t.diag(j) - sigma - b * b / p;
-      if (fabs(p) < pivmin) p = -pivmin;
-      neg += p < 0;
+  for (int o = 8; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    neg += __shfl_xor_sync(0xffffffffu, neg, o);
+  }
+  if (sub) neg = 0;
+  double p = 0.0, r = 0.0;   // the pivot; what it takes from the next one
+  if (sub < 2) {
+    const TwoEnds e(k, m, sub);
+    int j = e.j;
+    for (int i = 0; i < e.cnt; ++i, j += e.dj) {
+      p = t.diag(j) - sigma - r;
+      if (i == 0 && !e.l) p -= s;
+      if (i + 1 < e.cnt || !e.l) {
+        if (fabs(p) < pivmin) p = -pivmin;
+        neg += p < 0;
+        const int c = e.l ? j - 1 : j;
+        if (c + 1 < m) {
+          const double b = t.off(c);
+          r = b * b / p;
+        }
+      }
     }
   }
-  return __shfl_sync(0xffffffffu, neg, 0);
+  const double rc = __shfl_xor_sync(0xffffffffu, r, 1);
+  if (sub == 1 && m - k > 1) {   // the joined pivot
+    p -= rc;
+    if (fabs(p) < pivmin) p = -pivmin;
+    neg += p < 0;
+  }
+  return neg + __shfl_xor_sync(0xffffffffu, neg, 1);
 }
 
 __device__ double warp_normalize(double* z, int m) {
@@ -197,10 +251,18 @@ __device__ double ritz_pair_warp(const double* T, int ldt, int m, int k, int r, 
   // FP32 multisection: 32 shifts per round, keep [lo, hi] with count(lo) <= r < count(hi)
   float lo = (float)glo, hi = (float)ghi;
   const float pmin32 = (float)(tnorm * 1e-30) + 1e-30f;
+  float* d32 = (float*)piv;                      // FP32 copies: a conversion costs as much as an FP64 instruction
+  float* b32 = (float*)tz;
+  for (int j = lane; j < m; j += 32) {
+    d32[j] = (float)t.diag(j);
+    const float b = j < k ? (float)t.arrow(j) : j + 1 < m ? (float)t.off(j) : 0.f;
+    b32[j] = b * b;
+  }
+  __syncwarp();
   for (int round = 0; round < 8; ++round) {
     const float w = (hi - lo) / 33.0f;
     const float sig = lo + w * (float)(lane + 1);
-    const int cnt = inertia<float>(t, sig, pmin32);
+    const int cnt = inertia32(d32, b32, k, m, sig, pmin32);
     const unsigned below = __ballot_sync(0xffffffffu, cnt <= r);   // shifts still at or below lambda_r
     const int nb = __popc(below);                                   // counts are monotone in the shift
     const float nlo = nb > 0 ? __shfl_sync(0xffffffffu, sig, nb - 1) : lo;
@@ -232,8 +294,8 @@ __device__ double ritz_pair_warp(const double* T, int ldt, int m, int k, int r, 
   }
   // FP64 inertia on both sides: lambda must be the r-th eigenvalue (Sylvester)
   const double delta = 1e-9 * tnorm;
-  const int c_lo = inertia_warp(t, lambda - delta, pivmin);
-  const int c_hi = inertia_warp(t, lambda + delta, pivmin);
+  const int cnt2 = inertia2_warp(t, lambda - delta, lambda + delta, pivmin);
+  const int c_lo = __shfl_sync(0xffffffffu, cnt2, 0), c_hi = __shfl_sync(0xffffffffu, cnt2, 16);
   for (int j = lane; j < m; j += 32) zout[j] = z[j];
   return (c_lo <= r && c_hi >= r + 1 && lambda == lambda) ? lambda : NAN;
 }
