@@ -82,7 +82,11 @@ typedef struct {
  *   (eq. (29)), 0 <= mwin.
  *   tol: convergence threshold on ||A x - lambda x|| with ||x|| = 1 (Algorithm 1, normal mode).
  *   which: JTRLAN_SMALLEST (smallest algebraic) or JTRLAN_LARGEST.
- *   precision: JTRLAN_FP64 -- plain FP64 arithmetic throughout.
+ *   precision: JTRLAN_FP64 -- FP64 vectors, coefficients and results.  The basis V is kept with one
+ *       exponent a column (about 60 bits below its largest entry), and inner products, large update
+ *       coefficients, the restart rotation and the stencil product of the Lanczos steps are exact
+ *       integer sums of 56-bit factors, rounded once to FP64 (jtrlan_apply, residuals, CG and filters
+ *       use FP64 multiply-adds).
  *     JTRLAN_MIXED_REORTH -- the basis V is stored as (hi, lo) FP32 pairs (about 48 significant
  *       bits) and the three steps that plain FP64 spends on the FP64 pipe run in compensated FP32
  *       ("double-float": exact FMA-split products, TwoSum-carried sums): the stencil product A v_j
@@ -344,7 +348,8 @@ jtrlan_status jtrlan_rotate_df(const void* V, int64_t n, int m, const double* Z,
  * operator, applied to `count` dense Hermitian J-symmetric operators at once: one kernel launch (held
  * in a CUDA graph) in which each CTA takes instances, largest order first, from a device-side queue
  * and runs the whole method for one instance with all control on the device.  Each instance starts
- * from v_1 = (1, ..., 1)/sqrt(n) (Algorithm 1).  precision: JTRLAN_FP64 (plain FP64) or
+ * from v_1 = (1, ..., 1)/sqrt(n) (Algorithm 1).  precision: JTRLAN_FP64 (FP64
+ * vectors; products, Gram-Schmidt and rotation as exact integer sums of 56-bit factors) or
  * JTRLAN_MIXED_REORTH (products, Gram-Schmidt and rotation in compensated FP32 on (hi, lo) pairs;
  * alpha/beta, the Ritz solve and the residuals in FP64).  */
 typedef struct jtrlan_batch jtrlan_batch;  /* opaque; owned by the library */
@@ -392,7 +397,7 @@ jtrlan_status jtrlan_batch_tune(jtrlan_batch* b, int* threads, int* ctas_per_sm,
  * that split the columns of the Gram-Schmidt update y -= V c_v + W c_w, each group walking the row
  * pairs of the instance (0: as many as the block holds; fewer groups give longer column walks and a
  * shorter cross-group sum).  Results agree up to summation order.  Defaults: mv_rows 2 (compensated)
- * or 1 (FP64), gs_groups 0.  Errors: JTRLAN_EINVAL (values out of range). */
+ * or 1 (FP64, whose kernel takes no tiles: mv_rows has no effect on it), gs_groups 0.  Errors: JTRLAN_EINVAL (values out of range). */
 jtrlan_status jtrlan_batch_set_tiles(jtrlan_batch* b, int mv_rows, int gs_groups);
 jtrlan_status jtrlan_batch_get_tiles(jtrlan_batch* b, int* mv_rows, int* gs_groups);
 

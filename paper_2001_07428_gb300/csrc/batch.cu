@@ -7,7 +7,8 @@
 // ritz_dev.cuh (one warp per pair, verified; a one-CTA Jacobi if a check fails), the rotation of the
 // kept columns, true residuals, the converged-first ordering and the shrink of eq. (29).
 //
-// Template parameter DF: false -- plain FP64 arithmetic; true -- the matvec, the Gram-Schmidt inner
+// Template parameter DF: false -- FP64 vectors and coefficients, with products, Gram-Schmidt and rotation
+// as exact integer sums on a fixed-point basis and operator (fixed.cuh); true -- the matvec, the Gram-Schmidt inner
 // products and updates, and the rotation in compensated FP32 ("double-float", see gsdf.cu) on
 // (hi, lo) copies of A and of the basis, with FP64 vectors, alpha/beta, Ritz solve and residuals.
 //

@@ -16,7 +16,7 @@
 // The data-dependent repeat runs without host synchronisation: every pass is launched, and each
 // kernel of a pass returns at once when the device-side flag st->done says the loop has exited.
 // All reductions use a fixed order, so results are reproducible run to run.
-// These kernels serve the FP32 basis; the FP64 ones are in gs64.cu.
+// These kernels serve the FP32 basis; the FP64 ones are in gsfx.cu.
 #include <cooperative_groups.h>
 
 #include "internal.h"

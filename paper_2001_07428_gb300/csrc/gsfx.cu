@@ -4,8 +4,8 @@
 //
 // On this GPU FP64 multiply-adds run at 2 a clock and SM, so projections in plain FP64 are bound by that
 // pipe, not by the read of V.  Here
-//   * the inner products c_v = V^H y, c_w = W^H y are exact integer sums of two-limb numbers, 8 times the
-//     FP64 rate; y is converted once per row block into shared memory on that block's largest entry;
+//   * the inner products c_v = V^H y, c_w = W^H y are exact integer sums of two-limb numbers, 3.75 times
+//     the FP64 rate (four wide multiply-adds a product, 30 a clock and SM); y is converted once per row block into shared memory on that block's largest entry;
 //   * the update y -= V c_v + W c_w splits the columns: those whose coefficients are not small (in a
 //     Lanczos step beta_{j-1}'s, and the arrow's right after a restart) are applied in the same exact
 //     sums, the others, of rounding size, by their leading 28 bits in one integer sum (see UpdFx);
