@@ -1068,9 +1068,23 @@ __device__ void cta_ritz(const double* T, int ldt, int m, int k, int kk, int whi
         lambda = ztz / zz;
         if (lambda >= lo64 - slack && lambda <= hi64 + slack) sigma = lambda;
       }
-      const double delta = 1e-9 * tnorm;
-      const int c_lo = inertia_f64_serial(t, lambda - delta, pivmin);
-      const int c_hi = inertia_f64_serial(t, lambda + delta, pivmin);
+      lam[i] = lambda;
+    }
+  }
+  __syncthreads();
+  // the checks, a warp each: an FP64 instruction holds its warp's quarter of the SM, and the other quarters
+  // were idle (512 instances: compensated form 34.85 -> 34.33 ms, FP64 36.98 -> 36.63)
+  for (int task = w; task < 3 * groups; task += nw) {
+    const int g = task / 3, kind = task - 3 * g, i = 32 * g + lane;
+    if (i >= kk) continue;
+    const int r = (which == JTRLAN_LARGEST) ? m - 1 - i : i;
+    const double* z = zb + (size_t)g * 32 * m + lane;
+    const double lambda = lam[i], delta = 1e-9 * tnorm, pivmin = 1e-18 * tnorm + 1e-300;
+    bool good;
+    if (kind < 2) {
+      const int c = inertia_f64_serial(t, kind ? lambda + delta : lambda - delta, pivmin);
+      good = kind ? c >= r + 1 : c <= r;
+    } else {
       const double r2 = resid2_serial(t, z, lambda);
       double nn = 0.0;
       for (int q = 0; q < m; ++q) {
@@ -1078,11 +1092,9 @@ __device__ void cta_ritz(const double* T, int ldt, int m, int k, int kk, int whi
         Z[(size_t)i * m + q] = v;
         nn += v * v;
       }
-      lam[i] = lambda;
-      const bool good = c_lo <= r && c_hi >= r + 1 && lambda == lambda && sqrt(r2) <= 1e-11 * fmax(tmax, 1e-300) &&
-                        fabs(nn - 1.0) <= 1e-12;
-      if (!good) *ok = 0;
+      good = lambda == lambda && sqrt(r2) <= 1e-11 * fmax(tmax, 1e-300) && fabs(nn - 1.0) <= 1e-12;
     }
+    if (!good) *ok = 0;
   }
   __syncthreads();
 }
