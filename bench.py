@@ -92,9 +92,9 @@ NCU_TRAFFIC = {
     "matvec": dict(bytes=688.4e6, workload="stencil_24x24x24x48", kernel="stencil_df_cheb_kernel<float2, 32, 8> (middle step)",
                    source="paper_2001_07428_gb300/csrc/gsdf.cu",
                    sha256="c2b0951ee48049b03517a8577d49fbe4bbc4e41aec573dd88ab9d5cefbc4c298"),
-    "gs_step": dict(bytes=13.66e6, workload="stencil_8x8x8x8", kernel="gs_step_coop_kernel<double>",
-                    source="paper_2001_07428_gb300/csrc/gs.cu",
-                    sha256="25f4b188216fe6b311d90026b3e55046646e3a430ba0d7a2b9d8b809fdae98b5"),
+    "gs_step": dict(bytes=13.92e6, workload="stencil_8x8x8x8", kernel="gsfx_step_coop_kernel (a middle step)",
+                    source="paper_2001_07428_gb300/csrc/gsfx.cu",
+                    sha256="a5a48a8e2e49418e30b37d487dad125d4eeed03bcd3a571681030e739291fffc"),
 }
 
 
