@@ -1034,7 +1034,7 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
       LAUNCH(K_SHRINK, launch_store_cols(ph.V, ph.Vtmp, n, c->d_perm, k, m, c->vexp, c->kmax, s));
     else
       LAUNCH(K_SHRINK, launch_shrink<float>(ph.V, ph.Vtmp, n, c->d_perm, k, m, s));
-    if (ph.fx) c->nl[K_SHRINK] += 1;   // two kernels
+    if (ph.fx && k > 0) c->nl[K_SHRINK] += 1;   // two kernels
   }
   // carry the device counters of this phase into the next one
   c->work_base[0] = c->work[K_GS_FIRST];

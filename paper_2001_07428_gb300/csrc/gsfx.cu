@@ -722,9 +722,11 @@ inline unsigned col_grid(int64_t n) {
 
 cudaError_t launch_store_cols(void* V, const void* X, int64_t n, const int* perm, int k, int m, int* vexp, int* kmax,
                               cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(kmax, 0, (size_t)(k < 1 ? 1 : k) * sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  col_field_kernel<<<dim3(col_grid(n), k), 256, 0, s>>>((const double2*)X, n, perm, kmax);
+  if (k > 0) {   // k = 0: a restart that keeps v_{m+1} alone
+    cudaError_t e = cudaMemsetAsync(kmax, 0, (size_t)k * sizeof(int), s);
+    if (e != cudaSuccess) return e;
+    col_field_kernel<<<dim3(col_grid(n), k), 256, 0, s>>>((const double2*)X, n, perm, kmax);
+  }
   store_cols_kernel<<<dim3(col_grid(n), k < m ? k + 1 : k), 256, 0, s>>>((fxc*)V, (const double2*)X, n, perm, k, m, vexp,
                                                                         kmax);
   return cudaGetLastError();
