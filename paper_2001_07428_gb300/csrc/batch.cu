@@ -620,7 +620,7 @@ __device__ double cta_update_fx(const fxc* V, const double* coef, FxState& F, Fx
                                 long long* part, int gs_groups, int* ymax) {
   if (threadIdx.x < 32) {                                  // classify and convert the coefficients (j < 64)
     const int lane = threadIdx.x;
-    const float thr = (float)ynorm * (9.3132257e-10f / ((float)(j + 1) * (float)(j + 4)));
+    const int line = fx_line(ynorm, j);
     int fs = 0, fl = 0, g[3];
     bool large[3];
 #pragma unroll
@@ -630,10 +630,9 @@ __device__ double cta_update_fx(const fxc* V, const double* coef, FxState& F, Fx
       large[w] = false;
       if (i <= j) {
         const double* c = coef + 4 * i;
-        const float mx = fmaxf(fmaxf(fabsf((float)c[0]), fabsf((float)c[1])), fmaxf(fabsf((float)c[2]), fabsf((float)c[3])));
-        const int f = max(max(fx_field(c[0]), fx_field(c[1])), max(fx_field(c[2]), fx_field(c[3])));
+        const int mx = max(max(fx_high(c[0]), fx_high(c[1])), max(fx_high(c[2]), fx_high(c[3]))), f = mx >> 20;
         g[w] = f ? max(f + F.vexp[i] - 1023, 1) : 0;
-        large[w] = !(mx <= thr);
+        large[w] = mx > line;
         if (large[w]) fl = max(fl, g[w]);
         else fs = max(fs, g[w]);
       }

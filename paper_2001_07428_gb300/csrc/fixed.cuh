@@ -193,6 +193,20 @@ __device__ __forceinline__ double fx_warp_total(double v) {
   return fx_to_double(hi, lo, K - 1023 - 56 + 2);
 }
 
+// The high word of 2^-30 ynorm / ((j+1)(j+4)), the line between small and large coefficients of an update
+// (UpdFx in gsfx.cu).  A coefficient is compared by its own high word, fx_high: no FP64 instruction, and the
+// whole range of FP64 (as FP32 numbers both sides became infinite above 3.4e38, and every column small).  An
+// infinite or NaN ynorm gives 0, so that every nonzero coefficient is large.
+__device__ __forceinline__ int fx_high(double x) { return __double2hiint(x) & 0x7fffffff; }
+__device__ __forceinline__ int fx_line(double ynorm, int j) {
+  const int y = fx_high(ynorm), f = y >> 20;
+  if (f == 0x7ff) return 0;
+  const float t = __int_as_float(0x3f800000 | ((y & 0xfffff) << 3)) *   // the mantissa, in [1, 2)
+                  (9.3132257e-10f / ((float)(j + 1) * (float)(j + 4)));
+  const int b = __float_as_int(t), e = (b >> 23) - 127 + f;
+  return e < 1 ? 0 : (e << 20) | ((b >> 3) & 0xfffff);
+}
+
 __device__ __forceinline__ double fx_load(long long F, int K) { return fx_to_double(F >> 63, (unsigned long long)F, K - 1023 - 60); }
 
 }  // namespace jtr

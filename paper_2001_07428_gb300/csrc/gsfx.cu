@@ -162,25 +162,19 @@ __device__ __forceinline__ UpdFx upd_carve(unsigned char* p, int m) {
   return u;
 }
 
-// Classification and conversion of the coefficients; thr is the line between small and large in FP32 (the
-// comparison costs no FP64 instruction).
-__device__ __forceinline__ float upd_thr(double ynorm, int j) {
-  return (float)ynorm * (9.3132257e-10f / ((float)(j + 1) * (float)(j + 4)));
+// Classification and conversion of the coefficients; line: fx_line of the norm before the update.
+__device__ __forceinline__ int coef_high(const coef4& c) {
+  return max(max(fx_high(c.vr), fx_high(c.vi)), max(fx_high(c.wr), fx_high(c.wi)));
 }
-__device__ __forceinline__ int coef_field(const coef4& c) {
-  return max(max(fx_field(c.vr), fx_field(c.vi)), max(fx_field(c.wr), fx_field(c.wi)));
-}
-__device__ void classify(const GSArgs& a, float thr, UpdFx u) {
+__device__ void classify(const GSArgs& a, int line, UpdFx u) {
   const int j = a.j;
   __syncthreads();                                    // the last pass's readers are done
   if (threadIdx.x < 3) u.misc[threadIdx.x] = 0;
   __syncthreads();
   int fs = 0, fl = 0;
   for (int i = threadIdx.x; i <= j; i += kT) {
-    const coef4 c = a.coef[i];
-    const float m = fmaxf(fmaxf(fabsf((float)c.vr), fabsf((float)c.vi)), fmaxf(fabsf((float)c.wr), fabsf((float)c.wi)));
-    const bool large = !(m <= thr);
-    const int f = coef_field(c);
+    const int m = coef_high(a.coef[i]), f = m >> 20;
+    const bool large = m > line;
     const int g = f ? max(f + a.vexp[i] - 1023, 1) : 0;     // exponent field of the scaled coefficient
     u.list[i] = large ? 1 : 0;
     if (large) fl = max(fl, g);
@@ -499,7 +493,7 @@ __global__ void __launch_bounds__(kT, 1) gsfx_update_kernel(GSArgs a, int pass) 
   __syncthreads();
   if (s_skip) return;
   const UpdFx u = upd_carve(dyn + kBuf, a.m);
-  classify(a, upd_thr(a.st->nrm[pass - 1], a.j), u);             // ||y|| before this update
+  classify(a, fx_line(a.st->nrm[pass - 1], a.j), u);             // ||y|| before this update
   if (blockIdx.x == 0 && threadIdx.x == 0) a.st->units_update += (double)(a.j + 1) * (double)a.h;
   const int64_t p0 = (int64_t)blockIdx.x * a.rows_per_block;
   const int64_t p1 = min(p0 + (int64_t)a.rows_per_block, a.h);
@@ -603,7 +597,7 @@ gsfx_step_coop_kernel(GSArgs a, const double2* alpha_part, int n_alpha_part, int
       }
     }
     sync_all();                                           // coefficients complete
-    classify(a, upd_thr(bref, j), u);
+    classify(a, fx_line(bref, j), u);
     double* slot = nrm2 + (size_t)(pass & 1) * nblk;
     int* mslot = a.part_max + (size_t)(pass & 1) * nblk;
     {
