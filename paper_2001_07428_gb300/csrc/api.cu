@@ -173,6 +173,8 @@ struct jtrlan_ctx {
   bool tc_on = false;
   int* h_tcerr = nullptr;          // pinned copy of its error flag
   double fc = 0.0, fe = 1.0;       // filter window centre and half-width
+  void* links_fx = nullptr;        // p64.opfx's links, an optional copy (make_links_fx, drop_links)
+  bool links_tried = false;
   Profiler prof;
   double work_base[3] = {};        // device work counters carried across solve phases
   int fallback_base = 0;
@@ -184,10 +186,24 @@ struct jtrlan_ctx {
   std::vector<double> ev, res;
   jtrlan_stats stats{};
 
+  // Gives up the fixed-point links; false if there are none.
+  bool drop_links() {
+    if (!links_fx) return false;
+    cudaStreamSynchronize(stream);
+    cudaFree(links_fx);
+    links_fx = nullptr;
+    p64.fxmv = false;
+    return true;
+  }
   template <typename T_>
   jtrlan_status dalloc(T_** p, size_t bytes) {
     void* q = nullptr;
     cudaError_t e = cudaMalloc(&q, bytes ? bytes : 16);
+    if (e != cudaSuccess) cudaGetLastError();   // reported by the status
+    if (e == cudaErrorMemoryAllocation && drop_links()) {
+      e = cudaMalloc(&q, bytes ? bytes : 16);
+      if (e != cudaSuccess) cudaGetLastError();
+    }
     if (e != cudaSuccess) return fail(JTRLAN_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     owned.push_back(q);
     *p = (T_*)q;
@@ -206,6 +222,7 @@ struct jtrlan_ctx {
     cudaStreamSynchronize(stream);
     if (cg_group) cudaGraphExecDestroy(cg_group);
     for (void* p : owned) cudaFree(p);
+    if (links_fx) cudaFree(links_fx);
     for (void* p : owned_host) cudaFreeHost(p);
   }
 };
@@ -300,6 +317,39 @@ jtrlan_status setup_certify(jtrlan_ctx* c, const double* coeffs, int degree) {
   return JTRLAN_OK;
 }
 
+// The fixed-point links of the plain FP64 form (72 V numbers of 16 bytes) where they serve: the stencil product
+// of unfiltered Lanczos steps, not CG's.  They are the last buffer that jtrlan_create makes and are left out
+// where they would take more than half of the memory still free; every later need of the context that finds
+// none takes theirs (drop_links).  Without them the FP64 kernel serves.
+jtrlan_status make_links_fx(jtrlan_ctx* c) {
+  const OpDev& o = c->p64.op;
+  if (!c->p64.fx || c->invert || c->links_tried || o.kind != JTRLAN_STENCIL4D || c->n >= (int64_t)1 << 31)   // 32-bit sites and entries
+    return JTRLAN_OK;
+  c->links_tried = true;
+  const size_t bytes = (size_t)36 * o.vol * 16;
+  size_t room = 0, all = 0;
+  JT_CUDA(cudaMemGetInfo(&room, &all));
+  if (2 * bytes > room / 2) return JTRLAN_OK;
+  if (cudaMalloc(&c->links_fx, 2 * bytes + 2 * sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    c->links_fx = nullptr;
+    return JTRLAN_OK;
+  }
+  OpDev& d = c->p64.opfx;
+  d = o;
+  void *u = c->links_fx, *w = (char*)u + bytes;
+  int* k = (int*)((char*)w + bytes);
+  d.U = u;
+  d.W = w;
+  d.kfx = k;
+  JT_CUDA(launch_field(o.U, 36 * o.vol, k, c->stream));
+  JT_CUDA(launch_field(o.W, 36 * o.vol, k + 1, c->stream));
+  JT_CUDA(launch_links_fx(o.U, u, o.vol, k, c->stream));
+  JT_CUDA(launch_links_fx(o.W, w, o.vol, k + 1, c->stream));
+  c->p64.fxmv = true;   // its partials of alpha are fewer than the FP64 kernel's: 32 sites a block against 10.7
+  return JTRLAN_OK;
+}
+
 jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, void* stream, jtrlan_ctx** out) {
   JT_TRY(validate(op, prm));
   jtrlan_ctx* c = new (std::nothrow) jtrlan_ctx();
@@ -355,29 +405,6 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
     c->p64.fx = true;
     JT_TRY(make_phase(c->p64, sizeof(double2)));
     JT_TRY(c->dalloc(&c->p64.x, (size_t)c->n * sizeof(double2)));
-    if (op->kind == JTRLAN_STENCIL4D && c->n < (int64_t)1 << 31) {   // fixed-point links; 32-bit sites and entries
-      OpDev& d = c->p64.opfx;
-      d = o;
-      int* kfx = nullptr;
-      void* uw = nullptr;
-      const size_t bytes = (size_t)36 * o.vol * 16;
-      if (cudaMalloc(&uw, 2 * bytes) == cudaSuccess) {   // without room for them the FP64 kernel serves
-        c->owned.push_back(uw);
-        JT_TRY(c->dalloc(&kfx, 2 * sizeof(int)));
-        d.U = uw;
-        d.W = (char*)uw + bytes;
-        d.kfx = kfx;
-        JT_CUDA(launch_field(o.U, 36 * o.vol, kfx, c->stream));
-        JT_CUDA(launch_field(o.W, 36 * o.vol, kfx + 1, c->stream));
-        JT_CUDA(launch_links_fx(o.U, (void*)d.U, o.vol, kfx, c->stream));
-        JT_CUDA(launch_links_fx(o.W, (void*)d.W, o.vol, kfx + 1, c->stream));
-        c->p64.fxmv = true;
-      } else {
-        cudaGetLastError();
-      }
-      if (c->p64.fxmv && matvec_fx_blocks(d) > c->p64.alpha_nblk)
-        JT_TRY(c->dalloc(&c->p64.alpha_part, (size_t)matvec_fx_blocks(d) * sizeof(double2)));
-    }
   } else {  // double-float phase on the FP64 operator
     c->pdf.op = o;
     c->pdf.df = true;
@@ -562,6 +589,7 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
       return fail(JTRLAN_ENOTJSYM, buf);
     }
   }
+  if (!c->p64.filtered) JT_TRY(make_links_fx(c));
   JT_CUDA(cudaStreamSynchronize(c->stream));
   return JTRLAN_OK;
 }
@@ -1058,6 +1086,7 @@ jtrlan_status bounds_impl(jtrlan_ctx* c, int steps, double* lo, double* hi) {
   for (int t = 0; t < K_NTAGS; ++t) { c->prof.ms[t] = 0; c->nl[t] = 0; c->work[t] = 0; }
   JT_CUDA(cudaMemsetAsync(c->st, 0, sizeof(StepState), s));
   JT_CUDA(cudaMemsetAsync(c->T, 0, (size_t)ldt * ldt * sizeof(double), s));
+  JT_TRY(make_links_fx(c));   // a filtered context's only unfiltered steps
   const uint64_t seed = 0xb07d5ull;
   if (fp32) {
     LAUNCH(K_OTHER, launch_fill_random<float>(ph.V, n, seed, s));
@@ -1231,7 +1260,12 @@ jtrlan_status jtrlan_pairs(jtrlan_ctx* c, int with_partners, double* evals, void
         JT_CUDA(launch_gather_pairs(c->p64.Vtmp, c->d_perm, c->n, c->d_order, nev, with_partners, evecs, c->stream));
     } else {
       void* tmp = nullptr;
-      JT_CUDA(cudaMallocAsync(&tmp, bytes, c->stream));
+      cudaError_t e = cudaMallocAsync(&tmp, bytes, c->stream);
+      if (e == cudaErrorMemoryAllocation && c->drop_links()) {
+        cudaGetLastError();
+        e = cudaMallocAsync(&tmp, bytes, c->stream);
+      }
+      JT_CUDA(e);
       if (c->mixed)
         JT_CUDA(launch_gather_pairs_df(c->pdf.V, c->n, c->d_order, nev, with_partners, tmp, c->stream));
       else
