@@ -35,10 +35,10 @@ __device__ __forceinline__ int fx_field(double x) { return (__double2hiint(x) >>
 template <bool MinusZero>
 __device__ __forceinline__ fx2 fx_limbs(double x, int K) {
   const int hi = __double2hiint(x);
-  const uint32_t lo = (uint32_t)__double2loint(x);
   const int ex = (hi >> 20) & 0x7ff;
-  const uint32_t nz = (uint32_t)min(ex, 1);
-  const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
+  const uint32_t nz = (uint32_t)min(ex, 1), live = 0u - nz;
+  const uint32_t lo = (uint32_t)__double2loint(x) & live;
+  const uint32_t mh = (((uint32_t)hi & 0xfffffu) | 0x100000u) & live;   // K may be as low as 1
   const uint32_t th = __funnelshift_l(lo, mh, 11), tl = lo << 11;   // mantissa, left-aligned in 64 bits
   const uint32_t s = (uint32_t)(K - ex + 7);                        // >= 8; (th, tl) >> s is 2 floor(|x| 2^(55-e)) + a bit
   uint32_t h, g;

@@ -1,0 +1,81 @@
+"""The device helpers of csrc/fixed.cuh against exact Python integers (tests/cuda/fixed_probe.cu, compiled here)."""
+import ctypes
+import math
+import os
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2001_07428_gb300 import build as B
+    out = str(tmp_path_factory.mktemp("probe") / "fixed_probe.so")
+    subprocess.run([B.nvcc(), *B.ARCH, "-O3", "-std=c++17", "-shared", "-cudart", "shared", "-Xcompiler", "-fPIC",
+                    "-I", os.path.join(B.ROOT, "include"), "-o", out, os.path.join(HERE, "cuda", "fixed_probe.cu"),
+                    "-Xlinker", "-rpath," + B.cuda_lib_dir()], check=True)
+    torch.cuda.init()
+    return ctypes.CDLL(out)
+
+
+def _p(t):
+    return ctypes.c_void_p(t.data_ptr())
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+
+
+def _values(K):
+    """Doubles below 2^(K - 1023): full, short and far smaller significands, zeros, subnormals."""
+    rng = np.random.default_rng(K)
+    e = K - 1023
+    x = np.ldexp(rng.uniform(-1, 1, 400), e) * 2.0 ** -rng.integers(0, 64, 400).astype(float)
+    x = np.concatenate([x, [0.0, -0.0, 5e-324, -5e-324, 2.0 ** -1023, -(2.0 ** -1022 - 2.0 ** -1074)],
+                        np.ldexp([1.0 - 2.0 ** -53, -(1.0 - 2.0 ** -53), 0.5, -0.5, 2.0 ** -60, -(2.0 ** -60), 2.0 ** -61], e)])
+    return x[np.abs(x) < math.ldexp(1.0, e)] if e > -1021 else np.array([0.0, -0.0, 5e-324, -(2.0 ** -1023)])
+
+
+def _limbs(x, e):
+    if abs(x) < 2.0 ** -1022:
+        return 0, 0
+    f = 2 * int(abs(Fraction(x)) * Fraction(2) ** (55 - e)) + 1
+    f = -f if x < 0 else f
+    return f >> 28, f & ((1 << 28) - 1)
+
+
+@pytest.mark.parametrize("K", [1, 30, 1000, 1016, 1023, 1024, 1300])
+def test_limbs_and_store(probe, K):
+    x = _values(K)
+    d, n, e = _dev(x), len(x), K - 1023
+    lim = torch.empty((n, 2), dtype=torch.int32, device="cuda:0")
+    assert probe.probe_limbs(_p(d), n, K, _p(lim)) == 0
+    assert [tuple(r) for r in lim.cpu().tolist()] == [_limbs(v, e) for v in x]
+    if K < 1000:
+        return
+    F = torch.empty(n, dtype=torch.int64, device="cuda:0")
+    back = torch.empty(n, dtype=torch.float64, device="cuda:0")
+    assert probe.probe_store(_p(d), n, K, _p(F), _p(lim), _p(back)) == 0
+    for v, f, (h, l), b in zip(x, F.cpu().tolist(), lim.cpu().tolist(), back.cpu().tolist()):
+        q = Fraction(v) * Fraction(2) ** (60 - e)
+        want = math.floor(abs(q) + Fraction(1, 2)) * (-1 if q < 0 else 1) if abs(v) >= 2.0 ** -1022 else 0
+        assert f == want and (h, l) == ((f + 8) >> 32, ((f + 8) & 0xffffffff) >> 4)
+        assert b == float(Fraction(f) * Fraction(2) ** (e - 60))
+
+
+@pytest.mark.parametrize("cnt", [1, 2, 32, 33, 700])
+def test_warp_sums_of_zeros(probe, cnt):
+    """Zeros and subnormals count as zero."""
+    out = torch.empty(2, dtype=torch.float64, device="cuda:0")
+    for x in (np.zeros(cnt), -np.zeros(cnt), np.full(cnt, 5e-324)):
+        assert probe.probe_sum(_p(_dev(x)), cnt, _p(out)) == 0
+        assert out.cpu().tolist() == [0.0, 0.0]
