@@ -150,8 +150,10 @@ __device__ __forceinline__ double fx_lane_value(const FxAcc& a, int K) {
   return fx_to_double(H >> 36, ((unsigned long long)H << 28) | ((unsigned long long)t & 0x0fffffffull), K - 1023 - 84);
 }
 
-// Sum of the cnt doubles src[0], src[stride], ... over a warp, as limbs on the largest one's scale: off
-// from the exact sum by at most cnt 2^-56 of the largest.  Every lane gets the result.
+// Sum of the cnt doubles src[0], src[stride], ... over a warp, as limbs on the scale of the largest one (the
+// power of two above it): off from the exact sum by at most 2^-56 of the scale a term (its limbs) and a lane (the
+// bit that the 32 low limbs lose to fit their sum into 32 bits), before it is rounded once.  Every lane gets the
+// result.
 __device__ __forceinline__ double fx_warp_dsum(const double* src, int stride, int first, int cnt, int step) {
   int ex = 0;
   for (int i = first; i < cnt; i += step) ex = max(ex, fx_field(src[(int64_t)i * stride]));
@@ -170,13 +172,13 @@ __device__ __forceinline__ double fx_warp_dsum(const double* src, int stride, in
   }
   sh += sl >> 28;                                            // value (sh 2^28 + sl) 2^(K - 1023 - 56)
   const unsigned l = (unsigned)sl & 0x0fffffffu;
-  const unsigned w = __reduce_add_sync(0xffffffffu, l >> 2);
+  const unsigned w = __reduce_add_sync(0xffffffffu, l >> 1);
   const unsigned a0 = __reduce_add_sync(0xffffffffu, (unsigned)sh & 0x3ffffffu);
   const int a1 = __reduce_add_sync(0xffffffffu, (int)(sh >> 26));
-  const long long t = ((long long)a1 << 26) + (long long)a0;   // units 2^28; w in units 2^2
-  const unsigned long long lo = ((unsigned long long)t << 26) + w;
-  const long long hi = (t >> 38) + (lo < (unsigned long long)w ? 1 : 0);
-  return fx_to_double(hi, lo, K - 1023 - 56 + 2);
+  const long long t = ((long long)a1 << 26) + (long long)a0;   // units 2^28; w in units 2^1
+  const unsigned long long lo = ((unsigned long long)t << 27) + w;
+  const long long hi = (t >> 37) + (lo < (unsigned long long)w ? 1 : 0);
+  return fx_to_double(hi, lo, K - 1023 - 56 + 1);
 }
 
 // Sum of one double a lane, as fx_warp_dsum; every lane gets it.
@@ -185,12 +187,12 @@ __device__ __forceinline__ double fx_warp_total(double v) {
   if (ex == 0x7ff) return warp_sum(v);
   const int K = ex + 1;
   const fx2 t = fx_limbs<true>(v, K);
-  const unsigned w = __reduce_add_sync(0xffffffffu, (unsigned)t.l >> 2);          // units 2^2
+  const unsigned w = __reduce_add_sync(0xffffffffu, (unsigned)t.l >> 1);          // units 2^1
   const int a = __reduce_add_sync(0xffffffffu, t.h >> 14), b = __reduce_add_sync(0xffffffffu, t.h & 0x3fff);
   const long long hs = ((long long)a << 14) + b;                                  // units 2^28
-  const unsigned long long lo = ((unsigned long long)hs << 26) + w;
-  const long long hi = (hs >> 38) + (lo < (unsigned long long)w ? 1 : 0);
-  return fx_to_double(hi, lo, K - 1023 - 56 + 2);
+  const unsigned long long lo = ((unsigned long long)hs << 27) + w;
+  const long long hi = (hs >> 37) + (lo < (unsigned long long)w ? 1 : 0);
+  return fx_to_double(hi, lo, K - 1023 - 56 + 1);
 }
 
 // The high word of 2^-30 ynorm / ((j+1)(j+4)), the line between small and large coefficients of an update

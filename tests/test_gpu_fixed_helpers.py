@@ -79,3 +79,18 @@ def test_warp_sums_of_zeros(probe, cnt):
     for x in (np.zeros(cnt), -np.zeros(cnt), np.full(cnt, 5e-324)):
         assert probe.probe_sum(_p(_dev(x)), cnt, _p(out)) == 0
         assert out.cpu().tolist() == [0.0, 0.0]
+
+
+@pytest.mark.parametrize("cnt", [1, 2, 32, 33, 700])
+def test_warp_sum_error(probe, cnt):
+    """A term's limbs and a lane's dropped bit are each below 2^-56 of the scale, which is below twice the largest
+    term: 2^-54 of that a term; the result is rounded once."""
+    rng = np.random.default_rng(cnt)
+    out = torch.empty(2, dtype=torch.float64, device="cuda:0")
+    for x in (rng.standard_normal(cnt), rng.standard_normal(cnt) * 2.0 ** rng.integers(-80, 1, cnt).astype(float),
+              np.full(cnt, 1.0 - 2.0 ** -53)):
+        assert probe.probe_sum(_p(_dev(x)), cnt, _p(out)) == 0
+        top = np.abs(x).max()
+        for got, part in zip(out.cpu().tolist(), (x, x[:32])):
+            want = sum(map(Fraction, part), Fraction(0))
+            assert abs(Fraction(got) - want) <= len(part) * Fraction(2.0 ** -54) * Fraction(top) + abs(want) * Fraction(1, 2 ** 53)
