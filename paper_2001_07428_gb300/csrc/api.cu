@@ -137,7 +137,7 @@ struct jtrlan_ctx {
   double* part_dot = nullptr;
   double* part_nrm = nullptr;
   coef4* coef = nullptr;
-  int* vexp = nullptr;             // exponents of the basis columns (GSArgs)
+  int *vexp = nullptr, *vmin = nullptr;   // exponents of the basis columns (GSArgs)
   int* kmax = nullptr;             // scratch of launch_store_cols
   int* part_max = nullptr;
   StepState* st = nullptr;
@@ -555,6 +555,7 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
   JT_TRY(c->dalloc(&c->part_nrm, (size_t)2 * nblk_max * sizeof(double)));   // two slots (cooperative step)
   JT_TRY(c->dalloc(&c->coef, (size_t)(m + 1) * sizeof(coef4)));
   JT_TRY(c->dalloc(&c->vexp, (size_t)(m + 1) * sizeof(int)));
+  JT_TRY(c->dalloc(&c->vmin, (size_t)(m + 1) * sizeof(int)));
   JT_TRY(c->dalloc(&c->kmax, (size_t)(m + 1) * sizeof(int)));
   JT_TRY(c->dalloc(&c->part_max, (size_t)2 * nblk_max * sizeof(int)));
   JT_TRY(c->dalloc(&c->st, sizeof(StepState)));
@@ -869,7 +870,7 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
   a.V = ph.V; a.n = n; a.h = c->h; a.y = ph.y; a.part_dot = c->part_dot; a.part_nrm = c->part_nrm;
   a.coef = c->coef; a.st = c->st; a.T = c->T; a.ldt = ldt; a.m = m; a.nblk = c->gs_nblk;
   a.rows_per_block = c->gs_rpb;
-  a.vexp = c->vexp; a.part_max = c->part_max; a.x = (double2*)ph.x;
+  a.vexp = c->vexp; a.vmin = c->vmin; a.part_max = c->part_max; a.x = (double2*)ph.x;
   a.no_w = c->prm.plain_trlan ? 1 : 0;
   const double mv_units = ph.op.kind == JTRLAN_STENCIL4D ? (double)ph.op.vol : (double)c->h * (double)c->h;
   ev.assign(nev, 0.0);
@@ -1059,7 +1060,7 @@ jtrlan_status run_phase(jtrlan_ctx* c, Phase& ph, double tol, double tol_rel_tma
     if (ph.df)
       LAUNCH(K_SHRINK, launch_shrink_df(ph.V, ph.Vtmp, n, c->d_perm, k, m, s));  // and v_{k+1} = v_{m+1}
     else if (ph.fx)
-      LAUNCH(K_SHRINK, launch_store_cols(ph.V, ph.Vtmp, n, c->d_perm, k, m, c->vexp, c->kmax, s));
+      LAUNCH(K_SHRINK, launch_store_cols(ph.V, ph.Vtmp, n, c->d_perm, k, m, c->vexp, c->vmin, c->kmax, s));
     else
       LAUNCH(K_SHRINK, launch_shrink<float>(ph.V, ph.Vtmp, n, c->d_perm, k, m, s));
     if (ph.fx && k > 0) c->nl[K_SHRINK] += 1;   // two kernels
@@ -1095,13 +1096,13 @@ jtrlan_status bounds_impl(jtrlan_ctx* c, int steps, double* lo, double* hi) {
     LAUNCH(K_OTHER, launch_fill_random<double>(ph.x, n, seed, s));
     LAUNCH(K_OTHER, launch_normalize_col<double>(ph.x, n, c->part_nrm, c->gs_nblk, s));
     if (ph.df) LAUNCH(K_OTHER, launch_df_from_fp64(ph.x, ph.V, n, s));
-    else LAUNCH(K_OTHER, launch_store_cols(ph.V, ph.x, n, nullptr, 1, 0, c->vexp, c->kmax, s));
+    else LAUNCH(K_OTHER, launch_store_cols(ph.V, ph.x, n, nullptr, 1, 0, c->vexp, c->vmin, c->kmax, s));
   }
   GSArgs a{};
   a.V = ph.V; a.n = n; a.h = c->h; a.y = ph.y; a.part_dot = c->part_dot; a.part_nrm = c->part_nrm;
   a.coef = c->coef; a.st = c->st; a.T = c->T; a.ldt = ldt; a.m = c->m; a.nblk = c->gs_nblk;
   a.rows_per_block = c->gs_rpb;
-  a.vexp = c->vexp; a.part_max = c->part_max; a.x = (double2*)ph.x;
+  a.vexp = c->vexp; a.vmin = c->vmin; a.part_max = c->part_max; a.x = (double2*)ph.x;
   a.no_w = c->prm.plain_trlan ? 1 : 0;
   if (fp32) JT_TRY(lanczos_steps<float>(c, ph, a, 0, steps, false));
   else JT_TRY(lanczos_steps<double>(c, ph, a, 0, steps, false));
@@ -1171,7 +1172,7 @@ jtrlan_status solve_impl(jtrlan_ctx* c, jtrlan_stats* stats_out) {
   if (final.df) {   // normalised; stored as the basis's first column
     LAUNCH(K_OTHER, launch_df_from_fp64(final.x, final.V, n, s));
   } else {
-    LAUNCH(K_OTHER, launch_store_cols(final.V, final.x, n, nullptr, 1, 0, c->vexp, c->kmax, s));
+    LAUNCH(K_OTHER, launch_store_cols(final.V, final.x, n, nullptr, 1, 0, c->vexp, c->vmin, c->kmax, s));
     c->nl[K_OTHER] += 1;
   }
   jtrlan_stats s64{};

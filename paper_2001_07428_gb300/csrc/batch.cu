@@ -613,14 +613,17 @@ __device__ void cta_dot_fx(const fxc* V, const int* vexp, int64_t n, int64_t h, 
 }
 
 // y -= V c_v + W c_w; returns ||y||^2 (block-wide) and the high word of y's largest |component| in *ymax.
-// The columns are split as in gsfx.cu (UpdFx): those with a component above 2^-30 ||y|| / ((j+1)(j+4)) in
-// full, the others by the leading limb of V and 22 bits of the coefficient.  G groups of hp threads share
+// The columns are split as in gsfx.cu (UpdFx): those with a component above its line in full, the others by
+// the leading limb of V and 22 bits of the coefficient.  G groups of hp threads share
 // the small columns; group 0 adds their sums (part: 4 integers a thread), takes the large ones and y.
 __device__ double cta_update_fx(const fxc* V, const double* coef, FxState& F, FxCoef u, double* red, int64_t n, int64_t h, int j, double ynorm, double2* y,
                                 long long* part, int gs_groups, int* ymax) {
   if (threadIdx.x < 32) {                                  // classify and convert the coefficients (j < 64)
     const int lane = threadIdx.x;
     const int line = fx_line(ynorm, j);
+    int emin = 4096;
+    for (int i = lane; i <= j; i += 32) emin = min(emin, F.vexp[i]);
+    emin = __reduce_min_sync(0xffffffffu, emin);
     int fs = 0, fl = 0, g[3];
     bool large[3];
 #pragma unroll
@@ -632,7 +635,7 @@ __device__ double cta_update_fx(const fxc* V, const double* coef, FxState& F, Fx
         const double* c = coef + 4 * i;
         const int mx = max(max(fx_high(c[0]), fx_high(c[1])), max(fx_high(c[2]), fx_high(c[3]))), f = mx >> 20;
         g[w] = f ? max(f + F.vexp[i] - 1023, 1) : 0;
-        large[w] = mx > line;
+        large[w] = fx_large(mx, F.vexp[i] - emin, line);
         if (large[w]) fl = max(fl, g[w]);
         else fs = max(fs, g[w]);
       }

@@ -208,6 +208,10 @@ __device__ __forceinline__ int fx_line(double ynorm, int j) {
   const int b = __float_as_int(t), e = (b >> 23) - 127 + f;
   return e < 1 ? 0 : (e << 20) | ((b >> 3) & 0xfffff);
 }
+// Is a coefficient of high word m large in a column whose exponent is `spread` >= 0 above the least?
+__device__ __forceinline__ bool fx_large(int m, int spread, int line) {
+  return m != 0 && (unsigned)m + ((unsigned)spread << 20) > (unsigned)line;   // both below 2^31
+}
 
 __device__ __forceinline__ double fx_load(long long F, int K) { return fx_to_double(F >> 63, (unsigned long long)F, K - 1023 - 60); }
 

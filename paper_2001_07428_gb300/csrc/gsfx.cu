@@ -138,14 +138,19 @@ __device__ double dot_block(const GSArgs& a, int64_t p0, int64_t p1, int4* ys, i
 
 // ------------------------------------------------------------------ update
 // The coefficients in shared memory, prepared once per launch (every block alike).  Column i contributes
-// through its stored integers, so its coefficient is scaled by the column's 2^e.  A column is large when a
-// component of c_v or c_w exceeds 2^-30 ||y|| / ((j+1)(j+4)).  Large columns (list) are applied with both
-// limbs of both factors, on the scale 2^(KL - 1023) of the largest of them; the others with the leading
-// limb of V (28 bits) and 22 bits of the coefficient on the scale 2^(KS - 1023) of the line itself, in one
-// 64-bit sum: 2^28 2^22 times 4 (j+1) <= 2^12 terms stay below 2^63, and each term is off by less than
-// 2^-21 of the line times |v|, the whole sum by 2^-48 (j+1) ||y|| / ((j+1)(j+4)) |v| 2^-2 < 2^-50 / (j+4) of ||y|| |v|.
-// Rounding-size coefficients are about 2^-50 ||y||, far below the line for any j, so a step streams V
-// once at 16 multiply-adds a row pair and column.
+// through its stored integers, so its coefficient is scaled by the column's 2^e_i.  A column is large when a
+// component of c_v or c_w exceeds line 2^(e_min - e_i), line = 2^-30 ||y|| / ((j+1)(j+4)) and e_min the least
+// exponent of the columns: then no scaled coefficient of a small column exceeds line 2^e_min.  Large columns
+// (list) are applied with both limbs of both factors, on the scale 2^(KL - 1023) of the largest of them; the
+// others with the leading limb of V (28 bits) and 22 bits of the coefficient on the scale 2^(KS - 1023) of the
+// largest of theirs, at most 2 line 2^e_min, in one 64-bit sum: 2^28 2^22 times 4 (j+1) <= 2^12 terms stay below
+// 2^63.  A component of a coefficient is off by less than 2^-22 (1 + 2^-5) line, which over the columns makes
+// below 2^-50 / (j + 4) of ||y||; a component of V is off by less than 2^-28 of its column's scale, together below
+// 2^-56 rho / (j + 4) of ||y||, rho = 2^e_min sqrt(2n), the peak of the flattest column over its rms (below 16 for
+// a column of Gaussian entries).  Without the factor 2^(e_min - e_i) a small column with one entry near 1 set a
+// scale on which the coefficients of flat columns kept up to 11 bits fewer (n = 4M).
+// Rounding-size coefficients are about 2^-50 ||y||, far below the line for any j and for columns whose
+// exponents are a few apart, so a step streams V once at 16 multiply-adds a row pair and column.
 struct UpdFx {
   int4* sm;      // [m+1] small columns: c_v.re, c_v.im, c_w.re, c_w.im as integers (zero for a large one)
   int4* lg;      // [m+1][2] large columns: limbs of c_v (re, im), then of c_w
@@ -171,10 +176,11 @@ __device__ void classify(const GSArgs& a, int line, UpdFx u) {
   __syncthreads();                                    // the last pass's readers are done
   if (threadIdx.x < 3) u.misc[threadIdx.x] = 0;
   __syncthreads();
+  const int emin = a.vmin[j];
   int fs = 0, fl = 0;
   for (int i = threadIdx.x; i <= j; i += kT) {
     const int m = coef_high(a.coef[i]), f = m >> 20;
-    const bool large = m > line;
+    const bool large = fx_large(m, a.vexp[i] - emin, line);
     const int g = f ? max(f + a.vexp[i] - 1023, 1) : 0;     // exponent field of the scaled coefficient
     u.list[i] = large ? 1 : 0;
     if (large) fl = max(fl, g);
@@ -366,7 +372,10 @@ __device__ void normalize_block(const GSArgs& a, int64_t p0, int64_t p1, double 
   const double2* y = (const double2*)a.y;
   fxc* v = (fxc*)a.V + (int64_t)(a.j + 1) * a.n;
   const int K = fx_field(__hiloint2double(ymax + 1, 0) * inv) + 1;
-  if (p0 == 0 && threadIdx.x == 0) a.vexp[a.j + 1] = K;
+  if (p0 == 0 && threadIdx.x == 0) {
+    a.vexp[a.j + 1] = K;
+    a.vmin[a.j + 1] = min(a.vmin[a.j], K);
+  }
   const int64_t rows = p1 - p0;
   for (int64_t e = threadIdx.x; e < 2 * rows; e += kT) {
     const int64_t i = p0 + (e < rows ? e : e - rows + a.h);
@@ -662,10 +671,15 @@ __global__ void col_field_kernel(const double2* X, int64_t n, const int* perm, i
 // V[:, c] = X[:, perm[c]] (perm null: c) with the exponents kmax for c < k; V[:, k] = V[:, m] if k < m
 // (the restart's shrink of Algorithm 1).
 __global__ void store_cols_kernel(fxc* V, const double2* X, int64_t n, const int* perm, int k, int m, int* vexp,
-                                  const int* kmax) {
+                                  int* vmin, const int* kmax) {
   const int c = blockIdx.y;
   fxc* dst = V + (int64_t)c * n;
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, di = (int64_t)gridDim.x * blockDim.x;
+  if (i0 == 0) {
+    int e = c < k ? kmax[c] : vexp[m];
+    for (int i = 0; i < min(c, k); ++i) e = min(e, kmax[i]);
+    vmin[c] = e;
+  }
   if (c < k) {
     const double2* src = X + (int64_t)(perm ? perm[c] : c) * n;
     const int K = kmax[c];
@@ -714,15 +728,15 @@ inline unsigned col_grid(int64_t n) {
 
 }  // namespace
 
-cudaError_t launch_store_cols(void* V, const void* X, int64_t n, const int* perm, int k, int m, int* vexp, int* kmax,
-                              cudaStream_t s) {
+cudaError_t launch_store_cols(void* V, const void* X, int64_t n, const int* perm, int k, int m, int* vexp, int* vmin,
+                              int* kmax, cudaStream_t s) {
   if (k > 0) {   // k = 0: a restart that keeps v_{m+1} alone
     cudaError_t e = cudaMemsetAsync(kmax, 0, (size_t)k * sizeof(int), s);
     if (e != cudaSuccess) return e;
     col_field_kernel<<<dim3(col_grid(n), k), 256, 0, s>>>((const double2*)X, n, perm, kmax);
   }
   store_cols_kernel<<<dim3(col_grid(n), k < m ? k + 1 : k), 256, 0, s>>>((fxc*)V, (const double2*)X, n, perm, k, m, vexp,
-                                                                        kmax);
+                                                                        vmin, kmax);
   return cudaGetLastError();
 }
 

@@ -71,6 +71,7 @@ struct GSArgs {
   int rows_per_block;  // row pairs per block (multiple of 32)
   // the FP64 form (gsfx.cu), whose V is the fixed-point basis of fixed.cuh
   int* vexp;           // [m+1] K of the columns: |v| < 2^(K - 1023)
+  int* vmin;           // [m+1] the least K of columns 0..c
   int* part_max;       // [2][nblk] high words of the largest |component| of y
   double2* x;          // v_j in FP64 (the product's input), rewritten with v_{j+1} by the normalisation
 };
@@ -93,10 +94,10 @@ template <> cudaError_t launch_gs_update<double>(const GSArgs&, int, cudaStream_
 template <> cudaError_t launch_gs_dot<double>(const GSArgs&, int, cudaStream_t);
 template <> cudaError_t launch_gs_normalize<double>(const GSArgs&, cudaStream_t);
 // Columns of the fixed-point basis V (n x (m + 1)): store FP64 columns X[:, perm[c]] (perm null: c) as
-// V[:, 0..k) and, if k < m, V[:, m] as V[:, k]; load V[:, c] into x.  kmax: scratch
+// V[:, 0..k) and, if k < m, V[:, m] as V[:, k]; load V[:, c] into x.  vexp, vmin: GSArgs; kmax: scratch
 // of k ints.
-cudaError_t launch_store_cols(void* V, const void* X, int64_t n, const int* perm, int k, int m, int* vexp, int* kmax,
-                              cudaStream_t s);
+cudaError_t launch_store_cols(void* V, const void* X, int64_t n, const int* perm, int k, int m, int* vexp, int* vmin,
+                              int* kmax, cudaStream_t s);
 cudaError_t launch_load_col(const void* V, const int* vexp, int64_t n, int c, double2* x, cudaStream_t s);
 // out[:, c] = X[:, perm[order[c]]] and, if partners, out[:, nev + c] = J conj(X[:, perm[order[c]]]) (FP64).
 cudaError_t launch_gather_pairs(const void* X, const int* perm, int64_t n, const int* order, int nev, int partners,
