@@ -86,7 +86,12 @@ typedef struct {
  *       exponent a column (about 60 bits below its largest entry), and inner products, large update
  *       coefficients, the restart rotation and the stencil product of the Lanczos steps are exact
  *       integer sums of 56-bit factors, rounded once to FP64 (jtrlan_apply, residuals, CG and filters
- *       use FP64 multiply-adds).
+ *       use FP64 multiply-adds).  Such a factor is good to 2^-56 of the largest entry of its column, or
+ *       of its link field, where FP64 is good to 2^-53 of the entry itself: better for entries above 2^-3
+ *       of the largest, coarser for those far below.  The stencil product wants fixed-point copies
+ *       of the links, 1152 bytes a site: jtrlan_create makes them last, for unfiltered contexts, if they
+ *       take at most half of the memory still free (jtrlan_bounds does for a filtered one), and a later
+ *       allocation of the context that finds no room frees them; without them FP64 multiply-adds serve.
  *     JTRLAN_MIXED_REORTH -- the basis V is stored as (hi, lo) FP32 pairs (about 48 significant
  *       bits) and the three steps that plain FP64 spends on the FP64 pipe run in compensated FP32
  *       ("double-float": exact FMA-split products, TwoSum-carried sums): the stencil product A v_j
@@ -351,7 +356,10 @@ jtrlan_status jtrlan_rotate_df(const void* V, int64_t n, int m, const double* Z,
  * from v_1 = (1, ..., 1)/sqrt(n) (Algorithm 1).  precision: JTRLAN_FP64 (FP64
  * vectors; products, Gram-Schmidt and rotation as exact integer sums of 56-bit factors) or
  * JTRLAN_MIXED_REORTH (products, Gram-Schmidt and rotation in compensated FP32 on (hi, lo) pairs;
- * alpha/beta, the Ritz solve and the residuals in FP64).  */
+ * alpha/beta, the Ritz solve and the norms in FP64).  The products of the residual checks are those of
+ * the Lanczos steps: an operator of the FP64 form is rounded to 2^-57 of its largest entry when the batch
+ * is created, so a reported residual differs from that of the caller's blocks by up to n 2^-57 max|a|,
+ * and entries far below the largest (a graded matrix) are not seen to their own last bit. */
 typedef struct jtrlan_batch jtrlan_batch;  /* opaque; owned by the library */
 
 typedef struct {
@@ -393,10 +401,11 @@ jtrlan_status jtrlan_batch_set_shape(jtrlan_batch* b, int threads, int ctas_per_
 jtrlan_status jtrlan_batch_tune(jtrlan_batch* b, int* threads, int* ctas_per_sm, double* best_ms);
 
 /* Tile shapes of the persistent kernel.  mv_rows: rows of the product A v that a warp takes at once
- * (1 or 2; two rows share the loads of v).  gs_groups (compensated form only): the most thread groups
+ * (1 or 2; two rows share the loads of v).  gs_groups: the most thread groups
  * that split the columns of the Gram-Schmidt update y -= V c_v + W c_w, each group walking the row
  * pairs of the instance (0: as many as the block holds; fewer groups give longer column walks and a
- * shorter cross-group sum).  Results agree up to summation order.  Defaults: mv_rows 2 (compensated)
+ * shorter cross-group sum).  Results agree up to summation order (in the FP64 form, whose sums are exact,
+ * to the last bit; jtrlan_batch_tune leaves its gs_groups at 0).  Defaults: mv_rows 2 (compensated)
  * or 1 (FP64, whose kernel takes no tiles: mv_rows has no effect on it), gs_groups 0.  Errors: JTRLAN_EINVAL (values out of range). */
 jtrlan_status jtrlan_batch_set_tiles(jtrlan_batch* b, int mv_rows, int gs_groups);
 jtrlan_status jtrlan_batch_get_tiles(jtrlan_batch* b, int* mv_rows, int* gs_groups);
