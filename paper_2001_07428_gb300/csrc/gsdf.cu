@@ -1278,10 +1278,11 @@ static int df_cheb_blocks(const OpDev& op) { return (int)((op.vol + kChebSites -
 // Blocks of the fused step resident on an SM.  complex64 links: eight fill a large lattice best (24^3 x 48:
 // 237 us a step; six 242, five 261; 64 sites by four 242).  With few blocks for an SM the limit also spreads
 // them: the launch otherwise gives some SMs twice the blocks of others (from four to seven an SM on average a
-// step costs as much as eight), and the wider registers of four keep more loads in flight.  us a step at
-// 8 | 4 blocks an SM, the average count before:
-//   0.8 (8^4): 6.4 | 5.8, 1.7: 7.9 | 7.4, 2.5: 9.3 | 11.2, 3.4: 9.8 | 11.4, 4.2: 15.9 | 11.6, 5.1: 16.1 | 13.8,
-//   5.9: 16.2 | 16.3, 8.4: 19.1 | 18.1, 10: 22.0 | 22.1, 17: 32.6 | 33.5
+// step costs as much as eight, from eight to ten a second round of them), and the wider registers of four keep
+// more loads in flight.  us a step at 8 | 4 blocks an SM, the average count before:
+//   0.8 (8^4): 6.4 | 5.9, 1.5: 8.1 | 7.5, 2.1: 9.4 | 9.0, 3.0: 10.0 | 12.0, 4.3: 16.4 | 12.0, 5.0: 16.6 | 13.5,
+//   5.9: 17.0 | 17.1, 6.8: 17.0 | 17.2, 7.9: 17.0 | 18.1, 8.5: 20.7 | 18.8, 9.0: 21.2 | 20.7, 9.7: 22.5 | 21.2,
+//   10.4: 23.3 | 23.8, 11.8: 22.5 | 24.4, 13.5 (16^4): 26.6 | 26.6, 17: 34.2 | 34.7, 33: 62.1 | 65.8
 // (hi, lo) links want 142 registers (five blocks: 128) for the three columns of a direction at once; us a
 // step with one column at a time (64 sites by four, 80 registers) | now:
 //   0.8: 9.1 | 6.2, 1.7: 9.3 | 8.3, 2.5: 11.6 | 10.2, 3.4: 11.8 | 10.2, 4.2: 19.4 | 12.7, 6.7: 19.7 | 18.2,
@@ -1291,7 +1292,7 @@ static int df_cheb_per_sm(const OpDev& op) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int64_t nb = df_cheb_blocks(op), sm = nsm;
-  if (op.links32) return nb <= 2 * sm || (nb > 4 * sm && nb <= 6 * sm) ? 4 : 8;
+  if (op.links32) return nb <= 2 * sm || (nb > 4 * sm && nb <= 6 * sm) || (nb > 8 * sm && nb <= 10 * sm) ? 4 : 8;
   return nb <= 4 * sm ? 4 : 5;
 }
 
