@@ -515,8 +515,14 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
     int per = 0;
     if (!c->mixed) {
       JT_CUDA(gs_coop_occupancy<double>(m, &per));
-      // up to 32 tiles of rows go to eight blocks, one thread-block cluster (gsfx.cu)
-      if (per > 0) part(per, &c->coop_rpb, &c->coopfx, tiles <= 32 ? (tiles + 7) / 8 : 1);
+      // Up to 32 tiles of rows go to eight blocks, one thread-block cluster (gsfx.cu), unless m is large: then
+      // the columns are worth more SMs than the cheaper barriers are.  us a Lanczos step of a dense operator,
+      // cluster | a block a tile, m = 30, 60, 120, 200:
+      //    9 tiles: 38.2 | 40.7, 41.1 | 43.2, 48.2 | 48.4, 59.1 | 54.5
+      //   16 tiles: 47.5 | 51.0, 49.2 | 50.7, 57.8 | 54.7, 71.0 | 62.5
+      //   24 tiles: 58.3 | 61.3, 61.6 | 61.9, 73.1 | 66.7, 87.2 | 72.9
+      //   32 tiles: 77.1 | 83.7, 81.4 | 83.0, 95.8 | 87.8, 113.0 | 94.0
+      if (per > 0) part(per, &c->coop_rpb, &c->coopfx, tiles <= 32 && m <= 64 ? (tiles + 7) / 8 : 1);
     }
     if (prm->precision == JTRLAN_MIXED) {
       JT_CUDA(gs_coop_occupancy<float>(m, &per));
