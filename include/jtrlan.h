@@ -89,9 +89,10 @@ typedef struct {
  *       use FP64 multiply-adds).  Such a factor is good to 2^-56 of the largest entry of its column, or
  *       of its link field, where FP64 is good to 2^-53 of the entry itself: better for entries above 2^-3
  *       of the largest, coarser for those far below.  The stencil product wants fixed-point copies
- *       of the links, 1152 bytes a site: jtrlan_create makes them last, for unfiltered contexts, if they
- *       take at most half of the memory still free (jtrlan_bounds does for a filtered one), and a later
- *       allocation of the context that finds no room frees them; without them FP64 multiply-adds serve.
+ *       of the links, 1152 bytes a site: jtrlan_create makes them last, for unfiltered contexts (jtrlan_bounds
+ *       does for a filtered one), above 64 MB only if they take at most half of the memory still free, and
+ *       a later allocation of the context that finds no room frees them; without them FP64 multiply-adds
+ *       serve.
  *     JTRLAN_MIXED_REORTH -- the basis V is stored as (hi, lo) FP32 pairs (about 48 significant
  *       bits) and the three steps that plain FP64 spends on the FP64 pipe run in compensated FP32
  *       ("double-float": exact FMA-split products, TwoSum-carried sums): the stencil product A v_j

@@ -318,8 +318,8 @@ jtrlan_status setup_certify(jtrlan_ctx* c, const double* coeffs, int degree) {
 }
 
 // The fixed-point links of the plain FP64 form (72 V numbers of 16 bytes) where they serve: the stencil product
-// of unfiltered Lanczos steps, not CG's.  They are the last buffer that jtrlan_create makes and are left out
-// where they would take more than half of the memory still free; every later need of the context that finds
+// of unfiltered Lanczos steps, not CG's.  They are the last buffer that jtrlan_create makes and, above 64 MB, are
+// left out where they would take more than half of the memory still free; every later need of the context that finds
 // none takes theirs (drop_links).  Without them the FP64 kernel serves.
 jtrlan_status make_links_fx(jtrlan_ctx* c) {
   const OpDev& o = c->p64.op;
@@ -327,9 +327,11 @@ jtrlan_status make_links_fx(jtrlan_ctx* c) {
     return JTRLAN_OK;
   c->links_tried = true;
   const size_t bytes = (size_t)36 * o.vol * 16;
-  size_t room = 0, all = 0;
-  JT_CUDA(cudaMemGetInfo(&room, &all));
-  if (2 * bytes > room / 2) return JTRLAN_OK;
+  if (2 * bytes > (size_t)64 << 20) {   // asking takes about 0.1 ms
+    size_t room = 0, all = 0;
+    JT_CUDA(cudaMemGetInfo(&room, &all));
+    if (2 * bytes > room / 2) return JTRLAN_OK;
+  }
   if (cudaMalloc(&c->links_fx, 2 * bytes + 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     c->links_fx = nullptr;
@@ -560,8 +562,8 @@ jtrlan_status create_impl(const jtrlan_operator* op, const jtrlan_params* prm, v
   JT_TRY(c->dalloc(&c->part_dot, (size_t)(m + 1) * nblk_max * sizeof(coef4)));
   JT_TRY(c->dalloc(&c->part_nrm, (size_t)2 * nblk_max * sizeof(double)));   // two slots (cooperative step)
   JT_TRY(c->dalloc(&c->coef, (size_t)(m + 1) * sizeof(coef4)));
-  JT_TRY(c->dalloc(&c->vexp, (size_t)(m + 1) * sizeof(int)));
-  JT_TRY(c->dalloc(&c->vmin, (size_t)(m + 1) * sizeof(int)));
+  JT_TRY(c->dalloc(&c->vexp, (size_t)2 * (m + 1) * sizeof(int)));
+  c->vmin = c->vexp + m + 1;
   JT_TRY(c->dalloc(&c->kmax, (size_t)(m + 1) * sizeof(int)));
   JT_TRY(c->dalloc(&c->part_max, (size_t)2 * nblk_max * sizeof(int)));
   JT_TRY(c->dalloc(&c->st, sizeof(StepState)));
