@@ -181,7 +181,7 @@ ritz_check_kernel(const double* __restrict__ T, int ldt, int m, int k, int kk, i
 
 // ------------------------------------------------------------------ rotation V_m Z
 // out (n x kk complex) = V Z for the fixed-point basis (fixed.cuh), Z real: exact integer sums of two-limb
-// products, 16 a clock and SM against 2 FP64 multiply-adds.  A lane owns a complex row and four columns
+// products, 7.5 a clock and SM against 2 FP64 multiply-adds.  A lane owns a complex row and four columns
 // of Z (8 sums); the warps of a block share the row's loads through L1 and take other columns.  Z, scaled
 // by the columns' 2^e and converted on the scale of its largest entry per column, passes through shared
 // memory 64 rows at a time, the number of products a sum holds; then the sums leave for FP64.
